@@ -162,6 +162,20 @@ tpd_status tpd_decompose(void* A, int n, int dtype, const tpd_options* opt,
 tpd_status tpd_compose(void* C, int n, int dtype, double scale, const tpd_options* opt,
                        void* workspace, size_t workspace_bytes, void* stream);
 
+/* Out of place: as tpd_decompose / tpd_compose, reading the caller's matrix
+ * (device, only read) and leaving the result in another buffer (device, N*N
+ * elements; its contents on entry are ignored).  The first pass reads the one
+ * and writes the other, so no copy is made: a plan of P passes moves the
+ * matrix P times each way instead of P + 1.  Input and output have the
+ * alignment of tpd_decompose and are either the same buffer (then as in
+ * place) or do not overlap (INVALID_ARG otherwise).  Results are those of the
+ * in-place call on a copy, bit for bit.  Other arguments and errors as
+ * tpd_decompose / tpd_compose. */
+tpd_status tpd_decompose_to(const void* A, void* W, int n, int dtype, const tpd_options* opt,
+                            void* workspace, size_t workspace_bytes, void* stream);
+tpd_status tpd_compose_to(const void* C, void* A, int n, int dtype, double scale, const tpd_options* opt,
+                          void* workspace, size_t workspace_bytes, void* stream);
+
 /* End to end from host memory: copy A_host (N*N complex of `dtype`, host,
  * ideally pinned) into the caller's device buffer dev_A (device, N*N elements,
  * aligned as for tpd_decompose), decompose it in place, and copy the weights

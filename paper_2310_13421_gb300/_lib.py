@@ -32,7 +32,7 @@ SYMBOLS = (
     "tpd_convert_layout", "tpd_sum_squares", "tpd_partial_workspace_size", "tpd_partial_prepare",
     "tpd_decompose_partial", "tpd_nonzero_workspace_size", "tpd_nonzero_list", "tpd_sparse_workspace_size",
     "tpd_decompose_coo", "tpd_weyl_decompose", "tpd_weyl_compose", "tpd_gellmann_decompose",
-    "tpd_gellmann_compose",
+    "tpd_gellmann_compose", "tpd_decompose_to", "tpd_compose_to",
 )
 
 # size of the library's own scratch array used by tpd_decompose_noalloc
@@ -80,6 +80,10 @@ def load(path=None):
         lib.tpd_decompose.restype = i
         lib.tpd_compose.argtypes = [vp, i, i, ctypes.c_double, op, vp, sz, vp]
         lib.tpd_compose.restype = i
+        lib.tpd_decompose_to.argtypes = [vp, vp, i, i, op, vp, sz, vp]
+        lib.tpd_decompose_to.restype = i
+        lib.tpd_compose_to.argtypes = [vp, vp, i, i, ctypes.c_double, op, vp, sz, vp]
+        lib.tpd_compose_to.restype = i
         lib.tpd_tune_set.argtypes = [i, i, i, op]
         lib.tpd_tune_set.restype = i
         lib.tpd_tune_clear.argtypes = []
@@ -167,6 +171,16 @@ def tpd_decompose(A_ptr, n, dtype, opt=None, workspace=0, workspace_bytes=0, str
 def tpd_compose(C_ptr, n, dtype, scale, opt=None, workspace=0, workspace_bytes=0, stream=0):
     return int(load().tpd_compose(C_ptr, n, dtype, float(scale), _opt(opt), workspace or None,
                                   workspace_bytes, stream or None))
+
+
+def tpd_decompose_to(A_ptr, W_ptr, n, dtype, opt=None, workspace=0, workspace_bytes=0, stream=0):
+    return int(load().tpd_decompose_to(A_ptr or None, W_ptr or None, n, dtype, _opt(opt), workspace or None,
+                                       workspace_bytes, stream or None))
+
+
+def tpd_compose_to(C_ptr, A_ptr, n, dtype, scale, opt=None, workspace=0, workspace_bytes=0, stream=0):
+    return int(load().tpd_compose_to(C_ptr or None, A_ptr or None, n, dtype, float(scale), _opt(opt),
+                                     workspace or None, workspace_bytes, stream or None))
 
 
 def tpd_tune_set(n, dtype, precision, tuned=None):

@@ -46,6 +46,20 @@ def _check_device(t):
         raise ValueError("tensor must be contiguous (row-major)")
 
 
+def _target(A, inplace):
+    """(input, output) of a call on A.  In place: A itself.  Else a new output,
+    with A read where it is -- or, where A cannot be (a lazily conjugated or
+    negated view, memory not aligned to its elements, a tensor whose copy
+    autograd follows), a copy of it that is then worked on in place."""
+    if inplace:
+        return A, A
+    if (A.is_conj() or A.is_neg() or A.data_ptr() % A.element_size() or (A.requires_grad and torch.is_grad_enabled())
+            or torch.autograd.forward_ad._current_level >= 0):
+        out = A.clone()
+        return out, out
+    return A, torch.empty_like(A)
+
+
 def _stream(stream):
     s = stream if stream is not None else torch.cuda.current_stream()
     return s.cuda_stream
@@ -98,11 +112,11 @@ def decompose(A, *, inplace=False, precision=None, skip_zero=False, tile_bits=0,
     opt = make_options(precision, skip_zero, tile_bits, max_levels, variant, l2_chunk_mb)
     wsb = L.tpd_workspace_size(n, code, opt)
     with _enqueue(A.device, stream, A, workspace) as s:
-        out = A if inplace else A.clone()
+        src, out = _target(A, inplace)
         ws = workspace
         if wsb and (ws is None or ws.numel() < wsb):
             ws = torch.empty(wsb, dtype=torch.uint8, device=A.device)
-        st = L.tpd_decompose(out.data_ptr(), n, code, opt, ws.data_ptr() if wsb else 0, wsb, s)
+        st = L.tpd_decompose_to(src.data_ptr(), out.data_ptr(), n, code, opt, ws.data_ptr() if wsb else 0, wsb, s)
     _raise(st, "tpd_decompose")
     return out
 
@@ -116,11 +130,12 @@ def compose(C, *, scale=1.0, inplace=False, precision=None, skip_zero=False, til
     opt = make_options(precision, skip_zero, tile_bits, max_levels, variant)
     wsb = L.tpd_workspace_size(n, code, opt)
     with _enqueue(C.device, stream, C, workspace) as s:
-        out = C if inplace else C.clone()
+        src, out = _target(C, inplace)
         ws = workspace
         if wsb and (ws is None or ws.numel() < wsb):
             ws = torch.empty(wsb, dtype=torch.uint8, device=C.device)
-        st = L.tpd_compose(out.data_ptr(), n, code, float(scale), opt, ws.data_ptr() if wsb else 0, wsb, s)
+        st = L.tpd_compose_to(src.data_ptr(), out.data_ptr(), n, code, float(scale), opt, ws.data_ptr() if wsb else 0,
+                              wsb, s)
     _raise(st, "tpd_compose")
     return out
 

@@ -208,13 +208,13 @@ L2Chunks l2_chunks(const Plan& plan, const tpd_options* opt, bool off) {
   return r;
 }
 
-tpd_status run_single(bool dec, int arith, void* mat, const Plan& plan, int skip, double scale, void* ws,
+tpd_status run_single(bool dec, int arith, const void* src, void* mat, const Plan& plan, int skip, double scale, void* ws,
                       cudaStream_t s, const tpd_options* opt, const uint8_t* const* need) {
   record_event(opt, 0, s);
   if (plan.npass == 0) {
     SmallArgs a;
     std::memset(&a, 0, sizeof(a));
-    a.mat = mat; a.n = plan.n; a.skip_zero = skip;
+    a.mat = mat; a.src = src == mat ? nullptr : src; a.n = plan.n; a.skip_zero = skip;
     a.scale_mode = dec ? 0 : (scale == 1.0 ? 0 : 1);
     if (launch_small(arith, dec, a, 1, plan.n, s) != cudaSuccess) return TPD_ERR_CUDA;
     record_event(opt, 1, s);
@@ -227,6 +227,15 @@ tpd_status run_single(bool dec, int arith, void* mat, const Plan& plan, int skip
   // visits keep the "zero class" fill
   if ((skip || need) && lay.q_bytes && cudaMemsetAsync(w + lay.flags_bytes, kQFillByte, lay.q_bytes, s) != cudaSuccess)
     return TPD_ERR_CUDA;
+  // Zero skipping leaves all-zero tiles as they are; only the block fixed
+  // point's first pass carries them over to another buffer (in the other
+  // kernels the extra path costs registers, and a CTA per SM, on every call:
+  // fp32 64 -> 70, compensated 72 bytes of spills).  They work on a copy.
+  if (skip && src != mat && arith != kArithFixed) {
+    const size_t bytes = (size_t)arith_store_bytes(arith) << (2 * plan.n);
+    if (cudaMemcpyAsync(mat, src, bytes, cudaMemcpyDeviceToDevice, s) != cudaSuccess) return TPD_ERR_CUDA;
+    src = mat;
+  }
   int spow = 0;
   double sres = 1.0;
   if (!dec) split_scale(scale, &spow, &sres);
@@ -237,6 +246,7 @@ tpd_status run_single(bool dec, int arith, void* mat, const Plan& plan, int skip
     PassArgs a;
     std::memset(&a, 0, sizeof(a));
     a.mat = mat;
+    a.src = p == 0 && src != mat ? src : nullptr;
     a.skip_zero = skip;
     if (skip && p > 0) a.flags_in = reinterpret_cast<uint8_t*>(w + lay.flags_off[p]);
     if (skip && !last) a.flags_out = reinterpret_cast<uint8_t*>(w + lay.flags_off[p + 1]);
@@ -297,16 +307,20 @@ size_t single_ws(const Plan& plan, int arith, int skip) {
   return plan.npass > 1 ? layout_of(plan, arith, skip).total : 0;
 }
 
-tpd_status single(bool dec, void* mat, int n, int dtype, double scale, const tpd_options* opt_in, void* ws,
+// One matrix from src into mat: the same buffer (in place), or buffers that do not overlap.
+tpd_status single(bool dec, const void* src, void* mat, int n, int dtype, double scale, const tpd_options* opt_in, void* ws,
                   size_t ws_bytes, void* stream) {
   int prec = 0;
   tpd_status st = check_common(n, dtype, opt_in, &prec);
   if (st != TPD_OK) return st;
   const tpd_options eff = effective_options(n, dtype, prec, opt_in);
   const tpd_options* opt = &eff;
-  if (mat == nullptr) return TPD_ERR_INVALID_ARG;
+  if (mat == nullptr || src == nullptr) return TPD_ERR_INVALID_ARG;
   const size_t align = dtype == TPD_C128 ? 16 : 8;
-  if (reinterpret_cast<uintptr_t>(mat) % align) return TPD_ERR_MISALIGNED;
+  const uintptr_t m = reinterpret_cast<uintptr_t>(mat), sp = reinterpret_cast<uintptr_t>(src);
+  if (m % align || sp % align) return TPD_ERR_MISALIGNED;
+  const size_t bytes = align << (2 * n);
+  if (m != sp && m < sp + bytes && sp < m + bytes) return TPD_ERR_INVALID_ARG;
   if (!dec && (!std::isfinite(scale) || scale == 0.0)) return TPD_ERR_INVALID_ARG;
   const Plan* plan = get_plan(n, dtype, prec, opt);
   if (!plan) return TPD_ERR_INVALID_ARG;
@@ -317,7 +331,7 @@ tpd_status single(bool dec, void* mat, int n, int dtype, double scale, const tpd
   const size_t need = single_ws(*plan, arith, skip);
   if (need && (ws == nullptr || ws_bytes < need)) return TPD_ERR_WORKSPACE;
   if (ws && reinterpret_cast<uintptr_t>(ws) % 16) return TPD_ERR_MISALIGNED;
-  return run_single(dec, arith, mat, *plan, skip, scale, ws, static_cast<cudaStream_t>(stream), opt);
+  return run_single(dec, arith, src, mat, *plan, skip, scale, ws, static_cast<cudaStream_t>(stream), opt);
 }
 
 }  // namespace detail
@@ -344,12 +358,22 @@ size_t tpd_workspace_size(int n, int dtype, const tpd_options* opt_in) {
 
 tpd_status tpd_decompose(void* A, int n, int dtype, const tpd_options* opt, void* workspace,
                          size_t workspace_bytes, void* stream) {
-  return single(true, A, n, dtype, 1.0, opt, workspace, workspace_bytes, stream);
+  return single(true, A, A, n, dtype, 1.0, opt, workspace, workspace_bytes, stream);
+}
+
+tpd_status tpd_decompose_to(const void* A, void* W, int n, int dtype, const tpd_options* opt, void* workspace,
+                            size_t workspace_bytes, void* stream) {
+  return single(true, A, W, n, dtype, 1.0, opt, workspace, workspace_bytes, stream);
 }
 
 tpd_status tpd_compose(void* C, int n, int dtype, double scale, const tpd_options* opt, void* workspace,
                        size_t workspace_bytes, void* stream) {
-  return single(false, C, n, dtype, scale, opt, workspace, workspace_bytes, stream);
+  return single(false, C, C, n, dtype, scale, opt, workspace, workspace_bytes, stream);
+}
+
+tpd_status tpd_compose_to(const void* C, void* A, int n, int dtype, double scale, const tpd_options* opt,
+                          void* workspace, size_t workspace_bytes, void* stream) {
+  return single(false, C, A, n, dtype, scale, opt, workspace, workspace_bytes, stream);
 }
 
 tpd_status tpd_decompose_host(const void* A_host, void* W_host, void* dev_A, int n, int dtype,
@@ -363,7 +387,7 @@ tpd_status tpd_decompose_host(const void* A_host, void* W_host, void* dev_A, int
   const size_t bytes = ((size_t)1 << (2 * n)) * (dtype == TPD_C128 ? 16 : 8);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (cudaMemcpyAsync(dev_A, A_host, bytes, cudaMemcpyHostToDevice, s) != cudaSuccess) return TPD_ERR_CUDA;
-  st = single(true, dev_A, n, dtype, 1.0, opt, workspace, workspace_bytes, stream);
+  st = single(true, dev_A, dev_A, n, dtype, 1.0, opt, workspace, workspace_bytes, stream);
   if (st != TPD_OK) return st;
   if (cudaMemcpyAsync(W_host, dev_A, bytes, cudaMemcpyDeviceToHost, s) != cudaSuccess) return TPD_ERR_CUDA;
   return TPD_OK;

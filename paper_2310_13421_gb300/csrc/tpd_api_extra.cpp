@@ -216,7 +216,7 @@ tpd_status tpd_decompose_partial(void* A, int n, int dtype, const tpd_options* o
   const uint8_t* need[kMaxQubits];
   for (int p = 0; p < plan->npass; ++p) need[p] = reinterpret_cast<const uint8_t*>(w + lay.need_off[p]);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  st = run_single(true, arith, A, *plan, 0, 1.0, w + lay.run_off, s, &eff, plan->npass > 0 ? need : nullptr);
+  st = run_single(true, arith, A, A, *plan, 0, 1.0, w + lay.run_off, s, &eff, plan->npass > 0 ? need : nullptr);
   if (st != TPD_OK) return st;
   if (launch_gather(A, reinterpret_cast<const unsigned long long*>(w), count, (int)eb, weights, s) != cudaSuccess)
     return TPD_ERR_CUDA;

@@ -32,8 +32,8 @@ int sm_count();
 size_t single_ws(const Plan& plan, int arith, int skip);
 // classes of a pass (binary points it hands on): tiles x 2^(D-K)
 size_t class_count(const PassDesc& pd);
-// the passes of one matrix, in place; need: per-pass tile masks (partial decomposition) or nullptr
-tpd_status run_single(bool dec, int arith, void* mat, const Plan& plan, int skip, double scale, void* ws,
+// the passes of one matrix, from src (only read; may be mat) into mat; need: per-pass tile masks (partial decomposition) or nullptr
+tpd_status run_single(bool dec, int arith, const void* src, void* mat, const Plan& plan, int skip, double scale, void* ws,
                       cudaStream_t s, const tpd_options* opt, const uint8_t* const* need = nullptr);
 
 }  // namespace detail

@@ -243,7 +243,8 @@ __global__ void __launch_bounds__(kStdThreads, kOccLow) k_batch(const __grid_con
       if (sg.kind == kSegSmall) {
         // whole small matrices of the complex64 fixed-point form: the compensated kernel
         using SmallA = typename std::conditional<A::kFixed32, F32CArith, A>::type;
-        small_matrix<SmallA, kDec>(reinterpret_cast<Store*>(s_mat), sg.n, 0, bp.scale_mode, smem, tid, blockDim.x);
+        Store* const m = reinterpret_cast<Store*>(s_mat);
+        small_matrix<SmallA, kDec>(m, m, sg.n, 0, bp.scale_mode, smem, tid, blockDim.x);
       } else {
         for (int k = 0;; ++k) {
           const BatchSeg& sgk = bp.seg[vol_int(s_si)];

@@ -17,7 +17,9 @@ struct PassArgs {
   void* const* ptrs;          // nullptr: single matrix `mat`
   const int* items;
   long long tiles_per_mat;
-  void* mat;                  // matrix base (A::Store*), device
+  void* mat;                  // matrix base (A::Store*), device: the pass's output
+  const void* src;            // nullptr: in place; else (single matrix, first pass of an out-of-place call)
+                              // the caller's matrix, which is only read
   const uint8_t* flags_in;    // per tile of this pass: 0 = all zero, skip; nullptr = no skipping
   const uint8_t* need;        // per tile of this pass: 0 = feeds no requested weight (partial
                               // decomposition), skip; nullptr = every tile
@@ -60,7 +62,8 @@ struct SmallArgs {
   void* const* ptrs;          // batched: device array of matrix pointers (nullptr: use `mat`)
   const int* ns;              // batched: device array of n_i
   const int* items;           // batched: matrix index per CTA (nullptr: CTA i = matrix i)
-  void* mat;                  // single matrix
+  void* mat;                  // single matrix: output
+  const void* src;            // single matrix: nullptr (in place) or another matrix that is only read
   int n;                      // single matrix qubits
   int skip_zero;
   int scale_mode;             // compose: 0 scale 1, 1 scale 2^-n; decompose ignores
@@ -172,6 +175,9 @@ cudaError_t launch_small_c128(int arith, bool dec, const SmallArgs& args, int bl
 cudaError_t launch_pass_c64(int arith, bool dec, const PassDesc& pd, const PassArgs& args, long long ntiles_total,
                             cudaStream_t s);
 cudaError_t launch_small_c64(int arith, bool dec, const SmallArgs& args, int blocks, int n_max, cudaStream_t s);
+
+// bytes of a stored element
+inline int arith_store_bytes(int arith) { return (arith == kArithFixed || arith == kArithF64) ? 16 : 8; }
 
 // Persistent double-buffered fixed-point pass (D <= 12, single matrix, no
 // zero skipping): one CTA per SM, nsm = SM count.

@@ -446,6 +446,34 @@ __device__ __forceinline__ void load_tile(const G& pd, const void* matp, long lo
   for (int e = 0; e < kElems; ++e) raw[e] = ld_in<kCg>(mat + (g + reg_off(e, w0, w1, w2, w3)));
 }
 
+// The matrix a pass reads: its output `matp` itself (in place, and always for
+// the int64 sums of an earlier pass), or the input of an out-of-place call.
+// Reading the input here instead of copying it first saves one read and one
+// write of the matrix (GB300, n = 14 complex128: 6.16 -> 4.94 ms a call).
+// Read from the kernel's parameters where it is used: kept in registers
+// across the tile, the pointer spilled in the compensated first pass (n = 15:
+// 13.15 against 12.76 ms) and cost the batch 0.5 %.
+template <int kRole>
+__device__ __forceinline__ const void* pass_input(const PassArgs& args, const void* matp) {
+  if constexpr ((kRole & kRoleIntIn) != 0) return matp;
+  else return args.src != nullptr ? args.src : matp;
+}
+
+// An all-zero tile of an out-of-place call in the complex128 block fixed
+// point, which a pass otherwise leaves as it is: its elements (+-0) to their
+// positions in the output.
+template <class G>
+__device__ __forceinline__ void copy_tile(const G& pd, void* matp, long long base, int lane, int warp,
+                                          const double2 (&raw)[kElems]) {
+  const auto& s0 = pd.st[0];
+  double2* mat = reinterpret_cast<double2*>(matp);
+  const uint32_t g = (uint32_t)base + (uint32_t)thread_goff(pd, s0, lane, warp);
+  const uint32_t w0 = 1u << pd.gbit[s0.reg[0]], w1 = 1u << pd.gbit[s0.reg[1]];
+  const uint32_t w2 = 1u << pd.gbit[s0.reg[2]], w3 = 1u << pd.gbit[s0.reg[3]];
+#pragma unroll
+  for (int e = 0; e < kElems; ++e) mat[g + reg_off(e, w0, w1, w2, w3)] = raw[e];
+}
+
 // ============================================================== block fixed point
 //
 // A pass of the block fixed point reads IEEE numbers and writes IEEE numbers.
@@ -615,7 +643,7 @@ __device__ __noinline__ void ieee_tile(const PassDesc& pd, const PassArgs& args,
                                        int16_t* q_out, long long tile, long long base, uint32_t sbase, int nbase,
                                        unsigned char* smem, int lane, int warp) {
   double2 raw[kElems];
-  load_tile<kCg>(pd, matp, base, lane, warp, raw);
+  load_tile<kCg>(pd, (q_in != nullptr ? matp : pass_input<0>(args, matp)), base, lane, warp, raw);
   if (q_in != nullptr) {
     const Stage& s0 = pd.st[0];
     const uint32_t sb = sbase ^ src_thread(pd, s0, lane, warp);
@@ -761,7 +789,7 @@ __device__ __forceinline__ void fixed_tile(const G& pd, const PassArgs& args, vo
   auto prefetch_next = [&]() {
     if (pf_tile >= 0) {
       __syncthreads();
-      prefetch_tile(pd, matp, pf_tile, xbuf, lane, warp);
+      prefetch_tile(pd, pass_input<kRole>(args, matp), pf_tile, xbuf, lane, warp);
     }
   };
   constexpr bool kIntIn = (kRole & kRoleIntIn) != 0;
@@ -782,7 +810,7 @@ __device__ __forceinline__ void fixed_tile(const G& pd, const PassArgs& args, vo
     // ---- IEEE doubles: class maxima of the exponent fields
     double2 raw[kElems];
     if (inbuf) load_tile_smem(pd, inbuf, lane, warp, raw);
-    else load_tile<kCg>(pd, matp, base, lane, warp, raw);
+    else load_tile<kCg>(pd, pass_input<kRole>(args, matp), base, lane, warp, raw);
     if constexpr (kCl) cluster_wait();                   // the peer CTA is running
     __syncthreads();                                     // class slots cleared
     int lo;
@@ -801,7 +829,10 @@ __device__ __forceinline__ void fixed_tile(const G& pd, const PassArgs& args, vo
     slot_hi = hi;
     if ((args.skip_zero && !(tb & 1)) || (tb & 2)) {
       if (tb & 2)
-        ieee_tile<kDec, kCg, kCl>(raw_desc(pd), args, matp, q_in, q_out, tile, base, sbase, nbase, xbuf, lane, warp);
+        ieee_tile<kDec, kCg, kCl>(raw_desc(pd), args, matp, q_in, q_out, tile, base, sbase, nbase, xbuf, lane,
+                                  warp);
+      else if (args.src != nullptr)
+        copy_tile(pd, matp, base, lane, warp, raw);
       prefetch_next();
       return;                                            // (else all +-0: the outputs are zero already)
     }
@@ -822,7 +853,7 @@ __device__ __forceinline__ void fixed_tile(const G& pd, const PassArgs& args, vo
     longlong2 raw[kElems];
     int qs[kElems];
     if (inbuf) load_tile_smem(pd, inbuf, lane, warp, raw);
-    else load_tile<kCg>(pd, matp, base, lane, warp, raw);
+    else load_tile<kCg>(pd, pass_input<kRole>(args, matp), base, lane, warp, raw);
     {
       const uint32_t sb = sbase ^ src_thread(pd, s0, lane, warp);
       const uint32_t w0 = pd.src_w[s0.reg[0]], w1 = pd.src_w[s0.reg[1]], w2 = pd.src_w[s0.reg[2]],
@@ -847,7 +878,8 @@ __device__ __forceinline__ void fixed_tile(const G& pd, const PassArgs& args, vo
     slot_lo = lo;
     slot_hi = hi;
     if (tb & 2) {
-      ieee_tile<kDec, kCg, kCl>(raw_desc(pd), args, matp, q_in, q_out, tile, base, sbase, nbase, xbuf, lane, warp);
+      ieee_tile<kDec, kCg, kCl>(raw_desc(pd), args, matp, q_in, q_out, tile, base, sbase, nbase, xbuf, lane,
+                                warp);
       prefetch_next();
       return;
     }
@@ -958,7 +990,7 @@ __device__ __forceinline__ void fixed32_tile(const G& pd, const PassArgs& args, 
   const int ncls = 1 << (pd.D - pd.K);
   for (int i = threadIdx.x; i < ncls; i += nthr) cls[i] = 0;
   float2 raw[kElems];
-  load_tile<kCg>(pd, matp, base, lane, warp, raw);
+  load_tile<kCg>(pd, pass_input<0>(args, matp), base, lane, warp, raw);
   __syncthreads();                                       // class slots cleared
   int lo_unused;
   const uint32_t hmax = class_max<ExpSlot32>(pd, raw, cls, lane, warp, exp_f32, lo_unused);
@@ -1043,13 +1075,13 @@ __device__ __forceinline__ void pass_tile(const G& pd, const PassArgs& args, voi
     }
 
   if constexpr (A::kFixed) {
-    fixed_tile<kDec, kRole, kCg, kCl>(pd, args, matp, q_in, q_out, tile, base, sbase, nbase, nullptr, smem, red,
-                                      cls, lane, warp);
+    fixed_tile<kDec, kRole, kCg, kCl>(pd, args, matp, q_in, q_out, tile, base, sbase, nbase, nullptr, smem,
+                                      red, cls, lane, warp);
   } else if constexpr (A::kFixed32) {
     fixed32_tile<kDec, kCg>(pd, args, matp, base, nbase, smem, red, cls, lane, warp);
   } else {
     Store raw[kElems];
-    load_tile<kCg>(pd, matp, base, lane, warp, raw);
+    load_tile<kCg>(pd, pass_input<0>(args, matp), base, lane, warp, raw);
     if constexpr (kCl) cluster_wait();                   // the peer CTA is running
     if (args.skip_zero) {
       int nz = 0;
@@ -1167,14 +1199,15 @@ __global__ void __launch_bounds__(kStdThreads, 1)
   int* cls = red + kRedInts;
   long long tile = blockIdx.x;
   if (tile >= pd.ntiles) return;
-  prefetch_tile(pd, args.mat, tile, buf0, lane, warp);
+  const void* inp = pass_input<kRole>(args, args.mat);
+  prefetch_tile(pd, inp, tile, buf0, lane, warp);
   bool odd = false;
   for (; tile < pd.ntiles; tile += gridDim.x, odd = !odd) {
     unsigned char* cur = odd ? buf1 : buf0;
     unsigned char* spare = odd ? buf0 : buf1;
     const long long nxt = tile + gridDim.x;
     if (nxt < pd.ntiles) {
-      prefetch_tile(pd, args.mat, nxt, spare, lane, warp);
+      prefetch_tile(pd, inp, nxt, spare, lane, warp);
       cp_async_wait<1>();                 // this thread's copies of the current tile have landed
     } else {
       cp_async_wait<0>();
@@ -1189,8 +1222,8 @@ __global__ void __launch_bounds__(kStdThreads, 1)
         nbase += (int)pd.next_rest_w[j];
         sbase ^= pd.src_rest_w[j];
       }
-    fixed_tile<kDec, kRole>(pd, args, args.mat, args.q_in, args.q_out, tile, base, sbase, nbase, cur, cur, red, cls,
-                            lane, warp);
+    fixed_tile<kDec, kRole>(pd, args, args.mat, args.q_in, args.q_out, tile, base, sbase, nbase, cur, cur, red,
+                            cls, lane, warp);
     __syncthreads();                      // the current buffer is refilled next iteration
   }
 }
@@ -1213,7 +1246,8 @@ __global__ void __launch_bounds__(kStdThreads, kOccLow)
   int* cls = red + kRedInts;
   long long tile = blockIdx.x;
   if (tile >= pd.ntiles) return;
-  prefetch_tile(g, args.mat, tile, buf, lane, warp);
+  const void* inp = pass_input<kRole>(args, args.mat);
+  prefetch_tile(g, inp, tile, buf, lane, warp);
   for (; tile < pd.ntiles; tile += gridDim.x) {
     cp_async_wait<0>();
     __syncthreads();                      // the tile is in shared memory, everyone's copies included
@@ -1227,8 +1261,8 @@ __global__ void __launch_bounds__(kStdThreads, kOccLow)
         sbase ^= pd.src_rest_w[j];
       }
     const long long nxt = tile + gridDim.x;
-    fixed_tile<kDec, kRole>(g, args, args.mat, args.q_in, args.q_out, tile, base, sbase, nbase, buf, buf, red, cls,
-                            lane, warp, nxt < pd.ntiles ? nxt : -1);
+    fixed_tile<kDec, kRole>(g, args, args.mat, args.q_in, args.q_out, tile, base, sbase, nbase, buf, buf, red,
+                            cls, lane, warp, nxt < pd.ntiles ? nxt : -1);
   }
 }
 
@@ -1271,13 +1305,13 @@ __device__ __forceinline__ void small_levels(typename A::V* sm, int n, int tid, 
 // element (r, c) belongs to the class r xor c (its X-mask: every level keeps
 // it), and cls[x] holds that class's largest exponent field.
 template <class A, bool kDec>
-__device__ __forceinline__ void small_run(typename A::Store* mat, int n, int scale_mode, unsigned char* smem,
-                                          const int* cls, int tid, int nthr) {
+__device__ __forceinline__ void small_run(const typename A::Store* src, typename A::Store* mat, int n,
+                                          int scale_mode, unsigned char* smem, const int* cls, int tid, int nthr) {
   using V = typename A::V;
   V* sm = reinterpret_cast<V*>(smem);
   const int count = 1 << (2 * n), cmask = (1 << n) - 1;
   for (int i = tid; i < count; i += nthr) {
-    const typename A::Store x = mat[i];
+    const typename A::Store x = src[i];
     if constexpr (A::kFixed) {
       // x * 2^S with S = 1084 - n - E: headroom for the 2^n-term sums of n levels
       const int sb = 9 - n - max(cls[(i >> n) ^ (i & cmask)], 1);
@@ -1313,8 +1347,8 @@ __device__ __forceinline__ void small_run(typename A::Store* mat, int n, int sca
 // fallback for Inf/NaN), then small_run.  smem: 4^n elements of A::V, then
 // (block fixed point) 2^n class slots.
 template <class A, bool kDec>
-__device__ __forceinline__ void small_matrix(typename A::Store* mat, int n, int skip_zero, int scale_mode,
-                                             unsigned char* smem, int tid, int nthr) {
+__device__ __forceinline__ void small_matrix(const typename A::Store* src, typename A::Store* mat, int n,
+                                             int skip_zero, int scale_mode, unsigned char* smem, int tid, int nthr) {
   using Store = typename A::Store;
   const int count = 1 << (2 * n);
   if constexpr (A::kFixed) {
@@ -1324,7 +1358,7 @@ __device__ __forceinline__ void small_matrix(typename A::Store* mat, int n, int 
     __syncthreads();
     uint32_t hmax = 0, nzw = 0;
     for (int i = tid; i < count; i += nthr) {
-      const double2 x = mat[i];
+      const double2 x = src[i];
       const uint32_t ex = exp_f64(x);
       hmax = max(hmax, ex);
       nzw |= (uint32_t)__double2hiint(x.x) << 1 | (uint32_t)__double2loint(x.x) |
@@ -1333,16 +1367,20 @@ __device__ __forceinline__ void small_matrix(typename A::Store* mat, int n, int 
     }
     const int nz = __syncthreads_or(nzw != 0);
     const int inf = __syncthreads_or(hmax == 2047);
-    if (skip_zero && !nz) return;
-    if (inf) {
-      small_run<F64Arith, kDec>(mat, n, scale_mode, smem, nullptr, tid, nthr);
+    if (skip_zero && !nz) {
+      if (src != mat)
+        for (int i = tid; i < count; i += nthr) mat[i] = src[i];
       return;
     }
-    small_run<A, kDec>(mat, n, scale_mode, smem, cls, tid, nthr);
+    if (inf) {
+      small_run<F64Arith, kDec>(src, mat, n, scale_mode, smem, nullptr, tid, nthr);
+      return;
+    }
+    small_run<A, kDec>(src, mat, n, scale_mode, smem, cls, tid, nthr);
   } else {
     uint32_t nzw = 0;
     for (int i = tid; i < count; i += nthr) {
-      const Store x = mat[i];
+      const Store x = src[i];
       if constexpr (sizeof(Store) == 16) {
         nzw |= (uint32_t)__double2hiint(((const double2&)x).x) << 1 | (uint32_t)__double2loint(((const double2&)x).x) |
                (uint32_t)__double2hiint(((const double2&)x).y) << 1 | (uint32_t)__double2loint(((const double2&)x).y);
@@ -1351,8 +1389,12 @@ __device__ __forceinline__ void small_matrix(typename A::Store* mat, int n, int 
       }
     }
     const int nz = __syncthreads_or(nzw != 0);
-    if (skip_zero && !nz) return;
-    small_run<A, kDec>(mat, n, scale_mode, smem, nullptr, tid, nthr);
+    if (skip_zero && !nz) {
+      if (src != mat)
+        for (int i = tid; i < count; i += nthr) mat[i] = src[i];
+      return;
+    }
+    small_run<A, kDec>(src, mat, n, scale_mode, smem, nullptr, tid, nthr);
   }
 }
 
@@ -1365,8 +1407,9 @@ __global__ void __launch_bounds__(256) k_small(const SmallArgs args) {
   if (args.items) idx = args.items[idx];
   if (idx < 0) return;                     // bucketing found ns_dev inconsistent: touch nothing
   Store* mat = reinterpret_cast<Store*>(args.ptrs ? args.ptrs[idx] : args.mat);
+  const Store* src = args.src ? reinterpret_cast<const Store*>(args.src) : mat;
   const int n = args.ptrs ? args.ns[idx] : args.n;
-  small_matrix<A, kDec>(mat, n, args.skip_zero, args.scale_mode, smem, tid, nthr);
+  small_matrix<A, kDec>(src, mat, n, args.skip_zero, args.scale_mode, smem, tid, nthr);
 }
 
 }  // namespace tpd
