@@ -354,7 +354,8 @@ tpd_status tpd_decompose_coo(const int* rows, const int* cols, const void* value
  *           PLAIN (and DEFAULT for d = 5): IEEE fp64, rounded every level;
  *           complex64: fp32, rounded every level (FIXED and COMPENSATED are
  *           INVALID_ARG for complex64, FIXED for d = 5).
- * One kernel launch per qudit; no workspace; asynchronous on `stream`.
+ * complex128: one kernel launch per qudit; complex64: one per pass of up
+ * to 4, 3, 2, 2 levels for d = 2, 3, 4, 5.  No workspace; asynchronous on `stream`.
  * Errors: INVALID_ARG, MISALIGNED, CUDA. */
 tpd_status tpd_weyl_decompose(void* A, int n, int d, int dtype, const tpd_options* opt, void* stream);
 
@@ -394,7 +395,7 @@ tpd_status tpd_weyl_compose(void* C, int n, int d, int dtype, double scale, cons
  *           coefficients.
  *   opt     may be NULL; opt->precision DEFAULT or PLAIN (the same
  *           arithmetic); FIXED and COMPENSATED are INVALID_ARG.
- * One kernel launch per qudit; no workspace; asynchronous on `stream`.
+ * Launches as tpd_weyl_decompose; no workspace; asynchronous on `stream`.
  * Errors: INVALID_ARG, MISALIGNED, CUDA. */
 tpd_status tpd_gellmann_decompose(void* A, int n, int d, int dtype, const tpd_options* opt, void* stream);
 
@@ -406,6 +407,20 @@ tpd_status tpd_gellmann_decompose(void* A, int n, int d, int dtype, const tpd_op
  * tpd_gellmann_decompose. */
 tpd_status tpd_gellmann_compose(void* C, int n, int d, int dtype, double scale, const tpd_options* opt,
                                 void* stream);
+
+/* The qudit-basis calls out of place: the input (device, only read) and the
+ * result's buffer are the same (then as in place) or do not overlap
+ * (INVALID_ARG otherwise).  No copy is made: the first pass reads the one and
+ * writes the other.  Results, other arguments and errors as the in-place
+ * calls. */
+tpd_status tpd_weyl_decompose_to(const void* A, void* C, int n, int d, int dtype, const tpd_options* opt,
+                                 void* stream);
+tpd_status tpd_weyl_compose_to(const void* C, void* A, int n, int d, int dtype, double scale,
+                               const tpd_options* opt, void* stream);
+tpd_status tpd_gellmann_decompose_to(const void* A, void* G, int n, int d, int dtype, const tpd_options* opt,
+                                     void* stream);
+tpd_status tpd_gellmann_compose_to(const void* C, void* A, int n, int d, int dtype, double scale,
+                                   const tpd_options* opt, void* stream);
 
 /* Layout conversion, out of place.  RC is the layout every decomposition
  * leaves (see the conventions above); STRING puts the weight of

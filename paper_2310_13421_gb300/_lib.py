@@ -32,7 +32,8 @@ SYMBOLS = (
     "tpd_convert_layout", "tpd_sum_squares", "tpd_partial_workspace_size", "tpd_partial_prepare",
     "tpd_decompose_partial", "tpd_nonzero_workspace_size", "tpd_nonzero_list", "tpd_sparse_workspace_size",
     "tpd_decompose_coo", "tpd_weyl_decompose", "tpd_weyl_compose", "tpd_gellmann_decompose",
-    "tpd_gellmann_compose", "tpd_decompose_to", "tpd_compose_to",
+    "tpd_gellmann_compose", "tpd_decompose_to", "tpd_compose_to", "tpd_weyl_decompose_to",
+    "tpd_weyl_compose_to", "tpd_gellmann_decompose_to", "tpd_gellmann_compose_to",
 )
 
 # size of the library's own scratch array used by tpd_decompose_noalloc
@@ -110,6 +111,14 @@ def load(path=None):
         lib.tpd_gellmann_decompose.restype = i
         lib.tpd_gellmann_compose.argtypes = [vp, i, i, i, ctypes.c_double, op, vp]
         lib.tpd_gellmann_compose.restype = i
+        lib.tpd_weyl_decompose_to.argtypes = [vp, vp, i, i, i, op, vp]
+        lib.tpd_weyl_decompose_to.restype = i
+        lib.tpd_weyl_compose_to.argtypes = [vp, vp, i, i, i, ctypes.c_double, op, vp]
+        lib.tpd_weyl_compose_to.restype = i
+        lib.tpd_gellmann_decompose_to.argtypes = [vp, vp, i, i, i, op, vp]
+        lib.tpd_gellmann_decompose_to.restype = i
+        lib.tpd_gellmann_compose_to.argtypes = [vp, vp, i, i, i, ctypes.c_double, op, vp]
+        lib.tpd_gellmann_compose_to.restype = i
         lib.tpd_convert_layout.argtypes = [vp, vp, i, i, i, vp]
         lib.tpd_convert_layout.restype = i
         lib.tpd_sum_squares.argtypes = [vp, sz, i, vp, vp, sz, vp]
@@ -241,6 +250,22 @@ def tpd_gellmann_decompose(A, n, d, dtype, opt=None, stream=0):
 
 def tpd_gellmann_compose(C, n, d, dtype, scale, opt=None, stream=0):
     return int(load().tpd_gellmann_compose(C or None, n, d, dtype, float(scale), _opt(opt), stream or None))
+
+
+def tpd_weyl_decompose_to(A, C, n, d, dtype, opt=None, stream=0):
+    return int(load().tpd_weyl_decompose_to(A or None, C or None, n, d, dtype, _opt(opt), stream or None))
+
+
+def tpd_weyl_compose_to(C, A, n, d, dtype, scale, opt=None, stream=0):
+    return int(load().tpd_weyl_compose_to(C or None, A or None, n, d, dtype, float(scale), _opt(opt), stream or None))
+
+
+def tpd_gellmann_decompose_to(A, C, n, d, dtype, opt=None, stream=0):
+    return int(load().tpd_gellmann_decompose_to(A or None, C or None, n, d, dtype, _opt(opt), stream or None))
+
+
+def tpd_gellmann_compose_to(C, A, n, d, dtype, scale, opt=None, stream=0):
+    return int(load().tpd_gellmann_compose_to(C or None, A or None, n, d, dtype, float(scale), _opt(opt), stream or None))
 
 
 def tpd_convert_layout(src, dst, n, dtype, to_string, stream=0):

@@ -363,8 +363,8 @@ def weyl_decompose(A, d, *, inplace=False, precision=None, stream=None):
     n = _qudits(A, d)
     opt = make_options(precision)
     with _enqueue(A.device, stream, A) as s:
-        out = A if inplace else A.clone()
-        st = L.tpd_weyl_decompose(out.data_ptr(), n, int(d), _dtype_code(A), opt, s)
+        src, out = _target(A, inplace)
+        st = L.tpd_weyl_decompose_to(src.data_ptr(), out.data_ptr(), n, int(d), _dtype_code(A), opt, s)
     _raise(st, "tpd_weyl_decompose")
     return out
 
@@ -376,8 +376,8 @@ def weyl_compose(C, d, *, scale=1.0, inplace=False, precision=None, stream=None)
     n = _qudits(C, d)
     opt = make_options(precision)
     with _enqueue(C.device, stream, C) as s:
-        out = C if inplace else C.clone()
-        st = L.tpd_weyl_compose(out.data_ptr(), n, int(d), _dtype_code(C), float(scale), opt, s)
+        src, out = _target(C, inplace)
+        st = L.tpd_weyl_compose_to(src.data_ptr(), out.data_ptr(), n, int(d), _dtype_code(C), float(scale), opt, s)
     _raise(st, "tpd_weyl_compose")
     return out
 
@@ -392,8 +392,8 @@ def gellmann_decompose(A, d, *, inplace=False, precision=None, stream=None):
     n = _qudits(A, d)
     opt = make_options(precision)
     with _enqueue(A.device, stream, A) as s:
-        out = A if inplace else A.clone()
-        st = L.tpd_gellmann_decompose(out.data_ptr(), n, int(d), _dtype_code(A), opt, s)
+        src, out = _target(A, inplace)
+        st = L.tpd_gellmann_decompose_to(src.data_ptr(), out.data_ptr(), n, int(d), _dtype_code(A), opt, s)
     _raise(st, "tpd_gellmann_decompose")
     return out
 
@@ -405,8 +405,8 @@ def gellmann_compose(C, d, *, scale=1.0, inplace=False, precision=None, stream=N
     n = _qudits(C, d)
     opt = make_options(precision)
     with _enqueue(C.device, stream, C) as s:
-        out = C if inplace else C.clone()
-        st = L.tpd_gellmann_compose(out.data_ptr(), n, int(d), _dtype_code(C), float(scale), opt, s)
+        src, out = _target(C, inplace)
+        st = L.tpd_gellmann_compose_to(src.data_ptr(), out.data_ptr(), n, int(d), _dtype_code(C), float(scale), opt, s)
     _raise(st, "tpd_gellmann_compose")
     return out
 

@@ -10,8 +10,9 @@
 //     Omega_{a,b} = d^-1 sum_c omega^(-b c) A_{c+a, c}
 // (the d x d analogue of Eq. 4: for each shift a, a length-d DFT along the
 // block's a-th cyclic diagonal), and the levels commute.  On the GPU every
-// level is applied to all d x d blocks at once, in place: one launch per
-// qudit, each thread one block of d^2 elements in registers.  Omega_{a,b}
+// level is applied to all d x d blocks at once, in place; complex128: one
+// launch per qudit, each thread one block of d^2 elements in registers;
+// complex64: several levels per pass (tpd_qudit.cuh).  Omega_{a,b}
 // goes to the block position (row digit b, column digit a + b mod d), which
 // for d = 2 is where the Pauli decomposition puts I, X, Y, Z (with
 // W_{1,1} = XZ = -iY).  The composition inverts each level:
@@ -39,35 +40,13 @@
 #include <stdint.h>
 
 #include <cmath>
-#include <type_traits>
 
 #include "tpd.h"
 #include "tpd_arith.cuh"
+#include "tpd_weyl.cuh"
 
 namespace tpd {
 namespace {
-
-template <class T> struct C2;
-template <> struct C2<double> { using t = double2; };
-template <> struct C2<float> { using t = float2; };
-
-template <class T>
-struct Cx {
-  T re, im;
-};
-
-template <class T>
-__device__ __forceinline__ Cx<T> cadd(Cx<T> a, Cx<T> b) { return {a.re + b.re, a.im + b.im}; }
-template <class T>
-__device__ __forceinline__ Cx<T> csub(Cx<T> a, Cx<T> b) { return {a.re - b.re, a.im - b.im}; }
-// a * (wr + i wi), written without contraction into fused multiply-adds
-template <class T>
-__device__ __forceinline__ Cx<T> cmul(Cx<T> a, T wr, T wi) {
-  if constexpr (sizeof(T) == 8)
-    return {__dsub_rn(__dmul_rn(a.re, wr), __dmul_rn(a.im, wi)), __dadd_rn(__dmul_rn(a.re, wi), __dmul_rn(a.im, wr))};
-  else
-    return {__fsub_rn(__fmul_rn(a.re, wr), __fmul_rn(a.im, wi)), __fadd_rn(__fmul_rn(a.re, wi), __fmul_rn(a.im, wr))};
-}
 
 // Division of x < 2^32 by a divisor 0 < v < 2^32 fixed per launch: with
 // m = ceil(2^64 / v), floor(x m / 2^64) = floor(x / v) (the excess x (m -
@@ -99,46 +78,12 @@ __device__ __forceinline__ void weyl_block(uint32_t q, long long N, uint32_t s, 
   rs = (long long)s * N;
 }
 
-template <class T>
-struct Twiddles {
-  T re[8], im[8];     // omega^k, k < d
-  T h;                // sqrt(3) / 2 (d = 3)
-  T scale;            // factor applied to every output of this launch
-};
-
-// The d-point DFT of one class in the arithmetic T (y_b = sum_c omega^-bc x_c
-// for the decomposition, omega^+bc for the composition).
-template <class T, int D, bool kDec>
-__device__ __forceinline__ void dft_ieee(const Cx<T> (&x)[D], Cx<T> (&y)[D], const Twiddles<T>& tw) {
-  if constexpr (D == 3) {
-    const Cx<T> sm = cadd(x[1], x[2]), u = csub(x[1], x[2]);
-    const Cx<T> m = csub(x[0], Cx<T>{sm.re * T(0.5), sm.im * T(0.5)});
-    const Cx<T> hu = {u.re * tw.h, u.im * tw.h};
-    y[0] = cadd(x[0], sm);
-    // -i h u = (h u.im, -h u.re); the composition takes +i h u for y1
-    const Cx<T> mihu = {hu.im, -hu.re};
-    y[1] = kDec ? cadd(m, mihu) : csub(m, mihu);
-    y[2] = kDec ? csub(m, mihu) : cadd(m, mihu);
-  } else {
-#pragma unroll
-    for (int b = 0; b < D; ++b) {
-      Cx<T> acc = x[0];
-#pragma unroll
-      for (int c = 1; c < D; ++c) {
-        const int k = kDec ? (D - (b * c) % D) % D : (b * c) % D;
-        acc = cadd(acc, cmul(x[c], tw.re[k], tw.im[k]));
-      }
-      y[b] = acc;
-    }
-  }
-}
-
-// One qudit level on every d x d block: digit stride s (d^k for qudit n - k),
-// N = d^n, nblk = (N / D)^2 blocks.
-template <class T, int D, bool kDec>
-__global__ void __launch_bounds__(256) k_weyl_level(typename C2<T>::t* __restrict__ mat, long long N, long long s,
-                                                    long long nblk, const Twiddles<T> tw) {
-  using S = typename C2<T>::t;
+// One qudit level on every d x d block in IEEE fp64: digit stride s (d^k for
+// qudit n - k), N = d^n, nblk = (N / D)^2 blocks; src: the level's input, mat
+// itself but for the first level of an out-of-place call.
+template <int D, bool kDec>
+__global__ void __launch_bounds__(256) k_weyl_level(const double2* src, double2* mat, long long N, long long s,
+                                                    long long nblk, const Twiddles<double> tw) {
   const long long M = N / D;                 // other-digit combinations per row / column
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < nblk;
        q += (long long)gridDim.x * blockDim.x) {
@@ -146,37 +91,16 @@ __global__ void __launch_bounds__(256) k_weyl_level(typename C2<T>::t* __restric
     const long long R = (qr / s) * s * D + qr % s;   // digit k of the row set to 0
     const long long Cc = (qc / s) * s * D + qc % s;  // and of the column
     const long long base = R * N + Cc, rs = s * N;
-    Cx<T> in[D][D], out[D][D];
+    double2 in[D][D], out[D][D];
 #pragma unroll
     for (int r = 0; r < D; ++r)
 #pragma unroll
-      for (int c = 0; c < D; ++c) {
-        const S v = mat[base + r * rs + c * s];
-        in[r][c] = {v.x, v.y};
-      }
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-      // decomposition: x_c = A_{c+a, c} -> Omega_{a,b} at (b, a+b);
-      // composition: Omega_{a,b} at (b, a+b) -> A_{c+a, c}
-      Cx<T> x[D], y[D];
-#pragma unroll
-      for (int c = 0; c < D; ++c) x[c] = kDec ? in[(c + a) % D][c] : in[c][(a + c) % D];
-      dft_ieee<T, D, kDec>(x, y, tw);
-#pragma unroll
-      for (int b = 0; b < D; ++b) {
-        if (kDec) out[b][(a + b) % D] = y[b];
-        else out[(b + a) % D][b] = y[b];
-      }
-    }
+      for (int c = 0; c < D; ++c) in[r][c] = src[base + r * rs + c * s];
+    weyl_block_ieee<double, D, kDec>(in, out, tw);
 #pragma unroll
     for (int r = 0; r < D; ++r)
 #pragma unroll
-      for (int c = 0; c < D; ++c) {
-        S v;
-        v.x = out[r][c].re * tw.scale;
-        v.y = out[r][c].im * tw.scale;
-        mat[base + r * rs + c * s] = v;
-      }
+      for (int c = 0; c < D; ++c) mat[base + r * rs + c * s] = out[r][c];
   }
 }
 
@@ -209,7 +133,7 @@ __device__ __forceinline__ uint32_t exp_field(double2 v) {
 // (the composition's scale, on its last level) beyond the 1/d of the
 // decomposition.
 template <int D, bool kDec>
-__global__ void __launch_bounds__(256) k_weyl_level_fx(double2* __restrict__ mat, long long N, uint32_t s,
+__global__ void __launch_bounds__(256) k_weyl_level_fx(const double2* src, double2* mat, long long N, uint32_t s,
                                                        uint32_t nblk, const Div32 dM, const Div32 ds,
                                                        const Twiddles<double> tw, int out_pow2, double out_mul) {
   static_assert(D >= 2 && D <= 4, "fixed point for d = 2, 3, 4");
@@ -223,7 +147,7 @@ __global__ void __launch_bounds__(256) k_weyl_level_fx(double2* __restrict__ mat
 #pragma unroll
     for (int r = 0; r < D; ++r)
 #pragma unroll
-      for (int c = 0; c < D; ++c) in[r][c] = mat[base + r * rs + c * s];
+      for (int c = 0; c < D; ++c) in[r][c] = src[base + r * rs + c * s];
 #pragma unroll
     for (int a = 0; a < D; ++a) {
       double2 x[D];
@@ -313,26 +237,6 @@ __global__ void __launch_bounds__(256) k_weyl_level_fx(double2* __restrict__ mat
   }
 }
 
-// A cosine or sine within a few ulps of 0, +-1/2 or +-1 is that value
-// exactly, so quarter and sixth turns carry no rounding.
-double exact_if_near_half_integer(double v) {
-  const double h = std::nearbyint(2.0 * v) * 0.5;
-  return std::fabs(v - h) <= 4e-16 ? h : v;
-}
-
-template <class T>
-Twiddles<T> twiddles(int d, double scale) {
-  Twiddles<T> t{};
-  const double pi = 3.14159265358979323846;
-  for (int k = 0; k < d; ++k) {
-    t.re[k] = (T)exact_if_near_half_integer(std::cos(2.0 * pi * k / d));
-    t.im[k] = (T)exact_if_near_half_integer(std::sin(2.0 * pi * k / d));
-  }
-  t.h = (T)(std::sqrt(3.0) * 0.5);
-  t.scale = (T)scale;
-  return t;
-}
-
 // exponent of an exact power of two, else 0 with *resid = v
 int split_pow2(double v, double* resid) {
   int e = 0;
@@ -345,8 +249,9 @@ int split_pow2(double v, double* resid) {
   return 0;
 }
 
-template <class T, bool kDec>
-cudaError_t launch_levels(void* mat, int n, int d, double last_scale, bool fixed, cudaStream_t st) {
+template <bool kDec>
+cudaError_t launch_levels(const double2* src, double2* m, int n, int d, double last_scale, bool fixed,
+                          cudaStream_t st) {
   long long N = 1;
   for (int k = 0; k < n; ++k) N *= d;
   const long long nblk = (N / d) * (N / d);   // < 2^30: N <= 65536
@@ -358,51 +263,39 @@ cudaError_t launch_levels(void* mat, int n, int d, double last_scale, bool fixed
   long long grid = (nblk + 255) / 256;
   if (grid > 16ll * nsm) grid = 16ll * nsm;
   if (grid < 1) grid = 1;
-  using S = typename C2<T>::t;
+  const unsigned g = (unsigned)grid;
   long long s = 1;
   for (int k = 0; k < n; ++k, s *= d) {
     const Div32 ds = make_div32((uint32_t)s);
     // the decomposition's 1/d per level; the composition's scale on its last level
     const double sc = kDec ? 1.0 / d : (k == n - 1 ? last_scale : 1.0);
-    const Twiddles<T> tw = twiddles<T>(d, sc);
-    S* m = static_cast<S*>(mat);
-    if constexpr (std::is_same<T, double>::value) {
-      if (fixed && d <= 4) {
-        double resid = 1.0;
-        const int p2 = kDec ? 0 : split_pow2(sc, &resid);
-        double2* md = m;
-        const Twiddles<double>& twd = tw;
-        switch (d) {
-          case 2:
-            k_weyl_level_fx<2, kDec><<<(unsigned)grid, 256, 0, st>>>(md, N, (uint32_t)s, (uint32_t)nblk, dM, ds, twd,
-                                                                     p2, resid);
-            break;
-          case 3:
-            k_weyl_level_fx<3, kDec><<<(unsigned)grid, 256, 0, st>>>(md, N, (uint32_t)s, (uint32_t)nblk, dM, ds, twd,
-                                                                     p2, resid);
-            break;
-          default:
-            k_weyl_level_fx<4, kDec><<<(unsigned)grid, 256, 0, st>>>(md, N, (uint32_t)s, (uint32_t)nblk, dM, ds, twd,
-                                                                     p2, resid);
-            break;
-        }
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        continue;
+    const Twiddles<double> tw = twiddles<double>(d, sc);
+    if (fixed) {
+      double resid = 1.0;
+      const int p2 = kDec ? 0 : split_pow2(sc, &resid);
+      const uint32_t s32 = (uint32_t)s, nb = (uint32_t)nblk;
+      switch (d) {
+        case 2: k_weyl_level_fx<2, kDec><<<g, 256, 0, st>>>(src, m, N, s32, nb, dM, ds, tw, p2, resid); break;
+        case 3: k_weyl_level_fx<3, kDec><<<g, 256, 0, st>>>(src, m, N, s32, nb, dM, ds, tw, p2, resid); break;
+        default: k_weyl_level_fx<4, kDec><<<g, 256, 0, st>>>(src, m, N, s32, nb, dM, ds, tw, p2, resid); break;
+      }
+    } else {
+      switch (d) {
+        case 2: k_weyl_level<2, kDec><<<g, 256, 0, st>>>(src, m, N, s, nblk, tw); break;
+        case 3: k_weyl_level<3, kDec><<<g, 256, 0, st>>>(src, m, N, s, nblk, tw); break;
+        case 4: k_weyl_level<4, kDec><<<g, 256, 0, st>>>(src, m, N, s, nblk, tw); break;
+        default: k_weyl_level<5, kDec><<<g, 256, 0, st>>>(src, m, N, s, nblk, tw); break;
       }
     }
-    switch (d) {
-      case 2: k_weyl_level<T, 2, kDec><<<(unsigned)grid, 256, 0, st>>>(m, N, s, nblk, tw); break;
-      case 3: k_weyl_level<T, 3, kDec><<<(unsigned)grid, 256, 0, st>>>(m, N, s, nblk, tw); break;
-      case 4: k_weyl_level<T, 4, kDec><<<(unsigned)grid, 256, 0, st>>>(m, N, s, nblk, tw); break;
-      default: k_weyl_level<T, 5, kDec><<<(unsigned)grid, 256, 0, st>>>(m, N, s, nblk, tw); break;
-    }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    src = m;
   }
   return cudaSuccess;
 }
 
-tpd_status weyl_run(bool dec, void* A, int n, int d, int dtype, double scale, const tpd_options* opt, void* stream) {
-  if (A == nullptr || d < 2 || d > 5 || n < 1 || (dtype != TPD_C128 && dtype != TPD_C64)) return TPD_ERR_INVALID_ARG;
+tpd_status weyl_run(bool dec, const void* src, void* A, int n, int d, int dtype, double scale, const tpd_options* opt,
+                    void* stream) {
+  if (src == nullptr || A == nullptr || d < 2 || d > 5 || n < 1 || (dtype != TPD_C128 && dtype != TPD_C64)) return TPD_ERR_INVALID_ARG;
   // arithmetic: complex128 block fixed point (d <= 4) unless PLAIN is asked
   // for; complex64 fp32; FIXED for d = 5 or complex64 and COMPENSATED are
   // not offered
@@ -417,15 +310,19 @@ tpd_status weyl_run(bool dec, void* A, int n, int d, int dtype, double scale, co
   }
   if (!dec && (!std::isfinite(scale) || scale == 0.0)) return TPD_ERR_INVALID_ARG;
   const size_t align = dtype == TPD_C128 ? 16 : 8;
-  if (reinterpret_cast<uintptr_t>(A) % align) return TPD_ERR_MISALIGNED;
+  const uintptr_t m = reinterpret_cast<uintptr_t>(A), sp = reinterpret_cast<uintptr_t>(src);
+  if (m % align || sp % align) return TPD_ERR_MISALIGNED;
+  const size_t bytes = align * (size_t)(N * N);
+  if (m != sp && m < sp + bytes && sp < m + bytes) return TPD_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t e;
-  if (dtype == TPD_C128)
-    e = dec ? launch_levels<double, true>(A, n, d, 1.0, fixed, st)
-            : launch_levels<double, false>(A, n, d, scale, fixed, st);
-  else
-    e = dec ? launch_levels<float, true>(A, n, d, 1.0, false, st)
-            : launch_levels<float, false>(A, n, d, scale, false, st);
+  if (dtype == TPD_C128) {
+    const double2* in = static_cast<const double2*>(src);
+    double2* out = static_cast<double2*>(A);
+    e = dec ? launch_levels<true>(in, out, n, d, 1.0, fixed, st) : launch_levels<false>(in, out, n, d, scale, fixed, st);
+  } else {
+    e = weyl_c64(dec, static_cast<const float2*>(src), static_cast<float2*>(A), n, d, scale, st);
+  }
   return e == cudaSuccess ? TPD_OK : TPD_ERR_CUDA;
 }
 
@@ -435,12 +332,22 @@ tpd_status weyl_run(bool dec, void* A, int n, int d, int dtype, double scale, co
 extern "C" {
 
 tpd_status tpd_weyl_decompose(void* A, int n, int d, int dtype, const tpd_options* opt, void* stream) {
-  return tpd::weyl_run(true, A, n, d, dtype, 1.0, opt, stream);
+  return tpd::weyl_run(true, A, A, n, d, dtype, 1.0, opt, stream);
 }
 
 tpd_status tpd_weyl_compose(void* C, int n, int d, int dtype, double scale, const tpd_options* opt,
                             void* stream) {
-  return tpd::weyl_run(false, C, n, d, dtype, scale, opt, stream);
+  return tpd::weyl_run(false, C, C, n, d, dtype, scale, opt, stream);
+}
+
+tpd_status tpd_weyl_decompose_to(const void* A, void* C, int n, int d, int dtype, const tpd_options* opt,
+                                 void* stream) {
+  return tpd::weyl_run(true, A, C, n, d, dtype, 1.0, opt, stream);
+}
+
+tpd_status tpd_weyl_compose_to(const void* C, void* A, int n, int d, int dtype, double scale, const tpd_options* opt,
+                               void* stream) {
+  return tpd::weyl_run(false, C, A, n, d, dtype, scale, opt, stream);
 }
 
 }  // extern "C"
