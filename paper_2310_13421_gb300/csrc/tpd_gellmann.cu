@@ -56,16 +56,16 @@ __global__ void __launch_bounds__(256) k_gellmann_level(const double2* src, doub
     const uint32_t R = (qr / s) * s * D + qr % s;      // row with this qudit's digit 0
     const uint32_t C = (qc / s) * s * D + qc % s;      // column likewise
     const long long base = (long long)R * N + C, rs = (long long)s * N;
-    double2 x[D][D], y[D][D];
+    double2 x[D][D];
 #pragma unroll
     for (int r = 0; r < D; ++r)
 #pragma unroll
       for (int c = 0; c < D; ++c) x[r][c] = src[base + r * rs + (long long)c * s];
-    gm_block<double, D, kDec>(x, y, k);
+    gm_block<double, D, kDec>(x, k);
 #pragma unroll
     for (int r = 0; r < D; ++r)
 #pragma unroll
-      for (int c = 0; c < D; ++c) mat[base + r * rs + (long long)c * s] = y[r][c];
+      for (int c = 0; c < D; ++c) mat[base + r * rs + (long long)c * s] = x[r][c];
   }
 }
 

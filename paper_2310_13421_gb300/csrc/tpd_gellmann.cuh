@@ -59,61 +59,73 @@ struct GmConst {
   int scaled;      // scale != 1
 };
 
-// One block of a level: y from x.
-template <class T, int D, bool kDec, class S>
-__device__ __forceinline__ void gm_block(const S (&x)[D][D], S (&y)[D][D], const GmConst<T>& k) {
-  // off-diagonal pairs
-#pragma unroll
-  for (int j = 0; j < D; ++j)
-#pragma unroll
-    for (int i = j + 1; i < D; ++i) {
-      const S a = x[j][i], b = x[i][j];
-      if constexpr (kDec) {
-        y[j][i] = {ghalf(gadd(a.x, b.x)), ghalf(gadd(a.y, b.y))};
-        const T tr = ghalf(gsub(a.x, b.x)), ti = ghalf(gsub(a.y, b.y));
-        y[i][j] = {-ti, tr};                                   // i (a - b) / 2
-      } else {
-        y[j][i] = {gadd(a.x, b.y), gsub(a.y, b.x)};            // a - i b
-        y[i][j] = {gsub(a.x, b.y), gadd(a.y, b.x)};            // a + i b
-      }
-    }
-
-  // diagonal
+// The two parts of a level, on registers: an off-diagonal pair (a = x_jk,
+// b = x_kj, j < k) and the diagonal, each in place.
+template <bool kDec, class S>
+__device__ __forceinline__ void gm_pair(S& a, S& b) {
+  const S x = a, z = b;
   if constexpr (kDec) {
-    S P = x[0][0];                                             // running sum_{m<l} x_mm
+    a = {ghalf(gadd(x.x, z.x)), ghalf(gadd(x.y, z.y))};
+    const auto tr = ghalf(gsub(x.x, z.x)), ti = ghalf(gsub(x.y, z.y));
+    b = {-ti, tr};                                             // i (x - z) / 2
+  } else {
+    a = {gadd(x.x, z.y), gsub(x.y, z.x)};                      // x - i z
+    b = {gsub(x.x, z.y), gadd(x.y, z.x)};                      // x + i z
+  }
+}
+
+template <class T, int D, bool kDec, class S>
+__device__ __forceinline__ void gm_diag(S (&x)[D], const GmConst<T>& k) {
+  if constexpr (kDec) {
+    S P = x[0];                                                // running sum_{m<l} x_mm
 #pragma unroll
     for (int l = 1; l < D; ++l) {
-      const S xl = x[l][l];
+      const S xl = x[l];
       S lx = xl;                                               // l x_ll
       if (l == 2) lx = S{gtwice(xl.x), gtwice(xl.y)};
       if (l >= 3) lx = S{gmul(k.l[l], xl.x), gmul(k.l[l], xl.y)};
       if (l == 1)                                              // c_1 / 2 = 1/2 exactly
-        y[l][l] = {ghalf(gsub(P.x, lx.x)), ghalf(gsub(P.y, lx.y))};
+        x[l] = {ghalf(gsub(P.x, lx.x)), ghalf(gsub(P.y, lx.y))};
       else
-        y[l][l] = {gmul(k.hc[l], gsub(P.x, lx.x)), gmul(k.hc[l], gsub(P.y, lx.y))};
+        x[l] = {gmul(k.hc[l], gsub(P.x, lx.x)), gmul(k.hc[l], gsub(P.y, lx.y))};
       P = {gadd(P.x, xl.x), gadd(P.y, xl.y)};
     }
-    if constexpr (D == 2) y[0][0] = {ghalf(P.x), ghalf(P.y)};
-    else y[0][0] = {gmul(P.x, k.inv_d), gmul(P.y, k.inv_d)};
+    if constexpr (D == 2) x[0] = {ghalf(P.x), ghalf(P.y)};
+    else x[0] = {gmul(P.x, k.inv_d), gmul(P.y, k.inv_d)};
   } else {
-    const S y0 = x[0][0];
+    const S y0 = x[0];
     S Q = {T(0), T(0)};                                        // running sum_{l>m} c_l y_ll
 #pragma unroll
     for (int m = D - 1; m >= 1; --m) {
-      const S ym = x[m][m];
+      const S ym = x[m];
       // c_1 = 1 and 1 c_1 = 1 exactly: no multiply for m = 1
       const S cy = m == 1 ? ym : S{gmul(k.c[m], ym.x), gmul(k.c[m], ym.y)};
       const S lcy = m == 1 ? ym : S{gmul(k.lc[m], ym.x), gmul(k.lc[m], ym.y)};
-      y[m][m] = {gadd(y0.x, gsub(Q.x, lcy.x)), gadd(y0.y, gsub(Q.y, lcy.y))};
+      x[m] = {gadd(y0.x, gsub(Q.x, lcy.x)), gadd(y0.y, gsub(Q.y, lcy.y))};
       Q = {gadd(Q.x, cy.x), gadd(Q.y, cy.y)};
     }
-    y[0][0] = {gadd(y0.x, Q.x), gadd(y0.y, Q.y)};
+    x[0] = {gadd(y0.x, Q.x), gadd(y0.y, Q.y)};
   }
+}
+
+// A whole block of a level, in place.
+template <class T, int D, bool kDec, class S>
+__device__ __forceinline__ void gm_block(S (&x)[D][D], const GmConst<T>& k) {
+#pragma unroll
+  for (int j = 0; j < D; ++j)
+#pragma unroll
+    for (int i = j + 1; i < D; ++i) gm_pair<kDec>(x[j][i], x[i][j]);
+  S g[D];
+#pragma unroll
+  for (int m = 0; m < D; ++m) g[m] = x[m][m];
+  gm_diag<T, D, kDec>(g, k);
+#pragma unroll
+  for (int m = 0; m < D; ++m) x[m][m] = g[m];
   if (k.scaled) {
 #pragma unroll
     for (int r = 0; r < D; ++r)
 #pragma unroll
-      for (int c = 0; c < D; ++c) y[r][c] = {gmul(y[r][c].x, k.scale), gmul(y[r][c].y, k.scale)};
+      for (int c = 0; c < D; ++c) x[r][c] = {gmul(x[r][c].x, k.scale), gmul(x[r][c].y, k.scale)};
   }
 }
 
