@@ -298,6 +298,15 @@ tpd_status tpd_nonzero_list(const void* W, int n, int dtype, double tol, unsigne
                             void* weights, size_t capacity, unsigned long long* count, void* workspace,
                             size_t workspace_bytes, void* stream);
 
+/* The entries alone, from the counts that a tpd_nonzero_list call (with any
+ * capacity, 0 among them) on the same W, n, dtype and tol left in `workspace`:
+ * for callers that size their buffers by the count.  W must be unchanged.
+ * Blocks without entries are not read again.  Arguments and errors as
+ * tpd_nonzero_list. */
+tpd_status tpd_nonzero_write(const void* W, int n, int dtype, double tol, unsigned long long* strings,
+                             void* weights, size_t capacity, const void* workspace, size_t workspace_bytes,
+                             void* stream);
+
 /* Sparse input (the cost model of Sec. IV: m nonzero entries, p contributing
  * strings): the decomposition of a complex128 matrix given by its nonzero
  * entries, computed level by level as in Alg. 2 -- each entry of a CMW feeds

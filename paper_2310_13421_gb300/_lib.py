@@ -34,6 +34,7 @@ SYMBOLS = (
     "tpd_decompose_coo", "tpd_weyl_decompose", "tpd_weyl_compose", "tpd_gellmann_decompose",
     "tpd_gellmann_compose", "tpd_decompose_to", "tpd_compose_to", "tpd_weyl_decompose_to",
     "tpd_weyl_compose_to", "tpd_gellmann_decompose_to", "tpd_gellmann_compose_to",
+    "tpd_nonzero_write",
 )
 
 # size of the library's own scratch array used by tpd_decompose_noalloc
@@ -103,6 +104,8 @@ def load(path=None):
         lib.tpd_nonzero_workspace_size.restype = sz
         lib.tpd_nonzero_list.argtypes = [vp, i, i, ctypes.c_double, vp, vp, sz, vp, vp, sz, vp]
         lib.tpd_nonzero_list.restype = i
+        lib.tpd_nonzero_write.argtypes = [vp, i, i, ctypes.c_double, vp, vp, sz, vp, sz, vp]
+        lib.tpd_nonzero_write.restype = i
         lib.tpd_weyl_decompose.argtypes = [vp, i, i, i, op, vp]
         lib.tpd_weyl_decompose.restype = i
         lib.tpd_weyl_compose.argtypes = [vp, i, i, i, ctypes.c_double, op, vp]
@@ -234,6 +237,12 @@ def tpd_nonzero_workspace_size(n):
 def tpd_nonzero_list(W, n, dtype, tol, strings, weights, capacity, count, workspace, workspace_bytes, stream=0):
     return int(load().tpd_nonzero_list(W or None, n, dtype, float(tol), strings or None, weights or None, capacity,
                                        count or None, workspace or None, workspace_bytes, stream or None))
+
+
+def tpd_nonzero_write(W, n, dtype, tol, strings, weights, capacity, workspace, workspace_bytes, stream=0):
+    """Entries from the counts a tpd_nonzero_list call left in workspace."""
+    return int(load().tpd_nonzero_write(W or None, n, dtype, float(tol), strings or None, weights or None, capacity,
+                                        workspace or None, workspace_bytes, stream or None))
 
 
 def tpd_weyl_decompose(A, n, d, dtype, opt=None, stream=0):

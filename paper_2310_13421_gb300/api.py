@@ -294,8 +294,12 @@ def nonzero_list(W, *, tol=0.0, capacity=None, stream=None):
             cap = int(capacity)
         strings = torch.empty(max(cap, 1), dtype=torch.int64, device=W.device)
         weights = torch.empty(max(cap, 1), dtype=W.dtype, device=W.device)
-        st = L.tpd_nonzero_list(W.data_ptr(), n, code, tol, strings.data_ptr(), weights.data_ptr(), cap,
-                                count.data_ptr(), ws.data_ptr(), ws.numel(), s)
+        if capacity is None:                              # from the counts in ws
+            st = L.tpd_nonzero_write(W.data_ptr(), n, code, tol, strings.data_ptr(), weights.data_ptr(), cap,
+                                     ws.data_ptr(), ws.numel(), s)
+        else:
+            st = L.tpd_nonzero_list(W.data_ptr(), n, code, tol, strings.data_ptr(), weights.data_ptr(), cap,
+                                    count.data_ptr(), ws.data_ptr(), ws.numel(), s)
     _raise(st, "tpd_nonzero_list")
     if capacity is None:
         return strings[:cap], weights[:cap]

@@ -263,8 +263,27 @@ tpd_status tpd_nonzero_list(const void* W, int n, int dtype, double tol, unsigne
     return TPD_ERR_MISALIGNED;
   if (workspace == nullptr || workspace_bytes < nonzero_workspace_bytes(n)) return TPD_ERR_WORKSPACE;
   if (reinterpret_cast<uintptr_t>(workspace) % 256) return TPD_ERR_MISALIGNED;
-  if (launch_nonzero(W, n, (int)eb, tol, strings, weights, capacity, count, workspace,
-                     static_cast<cudaStream_t>(stream)) != cudaSuccess)
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (launch_nonzero_count(W, n, (int)eb, tol, count, workspace, s) != cudaSuccess) return TPD_ERR_CUDA;
+  if (capacity > 0 &&
+      launch_nonzero_write(W, n, (int)eb, tol, strings, weights, capacity, workspace, s) != cudaSuccess)
+    return TPD_ERR_CUDA;
+  return TPD_OK;
+}
+
+tpd_status tpd_nonzero_write(const void* W, int n, int dtype, double tol, unsigned long long* strings, void* weights,
+                             size_t capacity, const void* workspace, size_t workspace_bytes, void* stream) {
+  if (n < 1 || n > kMaxQubits || (dtype != TPD_C128 && dtype != TPD_C64)) return TPD_ERR_INVALID_ARG;
+  if (W == nullptr || !(tol >= 0.0) || (capacity > 0 && (strings == nullptr || weights == nullptr)))
+    return TPD_ERR_INVALID_ARG;
+  const size_t eb = dtype == TPD_C128 ? 16 : 8;
+  if (reinterpret_cast<uintptr_t>(W) % eb || reinterpret_cast<uintptr_t>(weights) % eb ||
+      reinterpret_cast<uintptr_t>(strings) % 8)
+    return TPD_ERR_MISALIGNED;
+  if (workspace == nullptr || workspace_bytes < nonzero_workspace_bytes(n)) return TPD_ERR_WORKSPACE;
+  if (reinterpret_cast<uintptr_t>(workspace) % 256) return TPD_ERR_MISALIGNED;
+  if (capacity > 0 && launch_nonzero_write(W, n, (int)eb, tol, strings, weights, capacity,
+                                           const_cast<void*>(workspace), static_cast<cudaStream_t>(stream)) != cudaSuccess)
     return TPD_ERR_CUDA;
   return TPD_OK;
 }

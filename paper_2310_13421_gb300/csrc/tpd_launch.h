@@ -140,11 +140,13 @@ constexpr int kCtrlDone = 4;
 cudaError_t launch_batch(int arith, bool dec, const BatchParams& bp, int* grid_out, cudaStream_t s);
 
 // Nonzero weights in string order (|re| > tol or |im| > tol; NaN kept): the
-// first `capacity` go to strings / weights, the number of all to *total.
+// number of all to *total and every block's to ws; then, from what the count
+// left in ws, the first `capacity` to strings / weights.
 size_t nonzero_workspace_bytes(int n);
-cudaError_t launch_nonzero(const void* W, int n, int elem_bytes, double tol, unsigned long long* strings,
-                           void* weights, unsigned long long capacity, unsigned long long* total, void* ws,
-                           cudaStream_t s);
+cudaError_t launch_nonzero_count(const void* W, int n, int elem_bytes, double tol, unsigned long long* total, void* ws,
+                                 cudaStream_t s);
+cudaError_t launch_nonzero_write(const void* W, int n, int elem_bytes, double tol, unsigned long long* strings,
+                                 void* weights, unsigned long long capacity, void* ws, cudaStream_t s);
 
 // Sparse (COO, complex128) decomposition into the list of nonzero weights,
 // sorted by string index; max_entries bounds the live entries of a level
