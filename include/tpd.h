@@ -355,16 +355,17 @@ tpd_status tpd_decompose_coo(const int* rows, const int* cols, const void* value
  *   dtype   TPD_C128 or TPD_C64.
  *   opt     may be NULL (defaults); only opt->precision is read:
  *           DEFAULT / FIXED: complex128 with d <= 4 in a block fixed point --
- *             the d elements each DFT combines (one cyclic diagonal of a
- *             block) on their own binary point in int64, the DFT exact for
- *             d = 2, 4 and with sqrt(3) rounded once on that grid for d = 3,
- *             one rounding to double per output and level (d = 2, 4 integer
- *             inputs: exact); classes meeting Inf/NaN in IEEE fp64;
+ *             the d^K elements that the K levels of a pass combine (one
+ *             digit-wise cyclic diagonal of a block) on their own binary point
+ *             in int64, the DFTs exact for d = 2, 4 and within a few units of
+ *             that grid for d = 3 (2^-56 of the largest element), one rounding
+ *             to double per output and pass (d = 2, 4 integer inputs: exact);
+ *             classes meeting Inf/NaN in IEEE fp64;
  *           PLAIN (and DEFAULT for d = 5): IEEE fp64, rounded every level;
  *           complex64: fp32, rounded every level (FIXED and COMPENSATED are
  *           INVALID_ARG for complex64, FIXED for d = 5).
- * complex128: one kernel launch per qudit; complex64: one per pass of up
- * to 4, 3, 2, 2 levels for d = 2, 3, 4, 5.  No workspace; asynchronous on `stream`.
+ * One kernel launch per pass of up to 4, 3, 2, 2 levels for d = 2, 3, 4,
+ * 5 (complex128 in IEEE fp64: per level).  No workspace; asynchronous on `stream`.
  * Errors: INVALID_ARG, MISALIGNED, CUDA. */
 tpd_status tpd_weyl_decompose(void* A, int n, int d, int dtype, const tpd_options* opt, void* stream);
 
@@ -404,7 +405,7 @@ tpd_status tpd_weyl_compose(void* C, int n, int d, int dtype, double scale, cons
  *           coefficients.
  *   opt     may be NULL; opt->precision DEFAULT or PLAIN (the same
  *           arithmetic); FIXED and COMPENSATED are INVALID_ARG.
- * Launches as tpd_weyl_decompose; no workspace; asynchronous on `stream`.
+ * One launch per qudit (complex64: per pass, as tpd_weyl_decompose); no workspace; asynchronous on `stream`.
  * Errors: INVALID_ARG, MISALIGNED, CUDA. */
 tpd_status tpd_gellmann_decompose(void* A, int n, int d, int dtype, const tpd_options* opt, void* stream);
 

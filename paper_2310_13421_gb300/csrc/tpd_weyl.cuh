@@ -107,4 +107,7 @@ inline Twiddles<T> twiddles(int d, double scale) {
 // n levels on complex64, several per pass (tpd_weyl_c64.cu)
 cudaError_t weyl_c64(bool dec, const float2* src, float2* mat, int n, int d, double last_scale, cudaStream_t st);
 
+// n levels on complex128 in block fixed point, d = 2, 3, 4 (tpd_weyl_fixed.cu)
+cudaError_t weyl_fixed(bool dec, const double2* src, double2* mat, int n, int d, double last_scale, cudaStream_t st);
+
 }  // namespace tpd
