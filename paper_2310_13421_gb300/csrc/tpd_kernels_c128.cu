@@ -22,15 +22,21 @@ cudaError_t ensure_smem_limit(const void* fn, size_t bytes) {
   return e;
 }
 
-int device_sm_count() {
+cudaError_t resident_ctas(const void* fn, int threads, size_t smem, long long* ctas) {
   static std::mutex mu;
-  static std::map<int, int> count;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+  static std::map<std::pair<const void*, int>, long long> known;   // (kernel, device) -> CTAs
+  int dev = 0, nsm = 0, per_sm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
   std::lock_guard<std::mutex> lk(mu);
-  int& c = count[dev];
-  if (c == 0 && cudaDeviceGetAttribute(&c, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) c = 0;
-  return c > 0 ? c : 1;
+  long long& c = known[std::make_pair(fn, dev)];
+  if (c == 0) {
+    if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem)) != cudaSuccess) return e;
+    c = (long long)nsm * (per_sm > 0 ? per_sm : 1);
+  }
+  *ctas = c;
+  return cudaSuccess;
 }
 
 cudaError_t launch_pass_fixed_dec(const PassDesc& pd, const PassArgs& args, long long ntiles_total, cudaStream_t s);

@@ -31,7 +31,10 @@ inline size_t class_slot_bytes(const PassDesc& pd) { return sizeof(int) << (pd.D
 PassKernel shape_kernel_fixed(bool dec, int shape, int role, int min_blocks);
 PassKernel shape_kernel_fixed_cl(bool dec, int shape, int role);   // two-CTA clusters
 PassKernel shape_kernel_fixed_pf(int shape, int role);              // persistent, prefetching
-int device_sm_count();                                              // of the current device (cached)
+// CTAs of a kernel that fit the current device at once, for its one block and
+// shared-memory size (asked once per kernel and device: the query costs as
+// much as a launch)
+cudaError_t resident_ctas(const void* fn, int threads, size_t smem, long long* ctas);
 PassKernel shape_kernel_c64(int arith, bool dec, int shape, int min_blocks);
 
 template <class A>
@@ -74,7 +77,7 @@ cudaError_t launch_pass_cl_t(const PassDesc& pd, const PassArgs& args, long long
       default: break;
     }
     if (!pd.rt_layout) {
-      const int shape = match_shape(pd);
+      const int shape = pd.shape;
       PassKernel sk = shape >= 0 ? shape_kernel_fixed_cl(kDec, shape, fixed_role(args)) : nullptr;
       if (sk != nullptr) kfn = sk;
     }
@@ -100,7 +103,7 @@ cudaError_t launch_pass_t(const PassDesc& pd, const PassArgs& args, long long nt
   const size_t smem_max = ((size_t)1 << dmax) * vbytes + kRedBytes + (kBlockFixed<A> ? sizeof(int) << (dmax - 1) : 0);
   PassKernel kfn = nullptr;
   if (!pd.rt_layout) {
-    const int shape = match_shape(pd);
+    const int shape = pd.shape;
     if constexpr (A::kFixed && kDec) {
       // one matrix, every tile: the persistent form that prefetches each
       // CTA's next tile while it finishes the current one
@@ -114,10 +117,9 @@ cudaError_t launch_pass_t(const PassDesc& pd, const PassArgs& args, long long nt
         cudaError_t e = ensure_smem_limit((const void*)pk, smem_pf_max);
         if (e != cudaSuccess) return e;
         if (ntiles_total <= 0) return cudaSuccess;
-        int per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pk, threads, smem_pf);
+        long long grid = 0;
+        e = resident_ctas((const void*)pk, threads, smem_pf, &grid);
         if (e != cudaSuccess) return e;
-        long long grid = (long long)device_sm_count() * (per_sm > 0 ? per_sm : 1);
         if (grid > ntiles_total) grid = ntiles_total;
         pk<<<(unsigned)grid, threads, smem_pf, s>>>(pd, args);
         return cudaGetLastError();

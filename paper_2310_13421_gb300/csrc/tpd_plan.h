@@ -86,6 +86,7 @@ struct PassDesc {
   int64_t next_rest_w[2 * kMaxQubits];
   int32_t min_blocks;        // CTAs per SM the pass kernel is compiled for (2 or 3); D = 13: 1 = one
                              // CTA of 512 threads, 2 = a two-CTA cluster of 256 (complex128)
+  int32_t shape;             // the compiled shape (tpd_shape.h) this layout equals, or -1
   int32_t rt_layout;         // 1: run the kernel that reads the layout from this descriptor even
                              // where a compiled shape (tpd_shape.h) matches it
   // Block fixed point: the *class* of a tile position.  A pass only ever adds

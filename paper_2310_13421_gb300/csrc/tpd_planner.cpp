@@ -384,6 +384,7 @@ bool build_plan(int n, int dtype, int precision, int tile_bits_opt, int max_leve
       if (pd.st[s].npair != 2 || pd.st[s].nshfl != 0) pairs_only = false;
     const bool two_c64 = pairs_only && precision == 3 && pd.D < 12;
     const bool three = dtype == 1 && precision >= 2 && !two_c64;
+    pd.shape = match_shape(pd);
     pd.min_blocks = pd.D > 12 ? (dtype == 0 ? 2 : 1) : (three ? kOccHigh : kOccLow);
   }
   return true;
@@ -412,7 +413,7 @@ std::string describe_plan(const Plan& plan) {
       s += buf;
     }
     // the compiled tile layout (tpd_shape.h) this pass's layout equals, or -1
-    std::snprintf(buf, sizeof(buf), " shape=%d", match_shape(pd));
+    std::snprintf(buf, sizeof(buf), " shape=%d", pd.shape);
     s += buf;
     for (int si = 0; si < pd.nstage; ++si) {
       const Stage& st = pd.st[si];
