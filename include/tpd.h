@@ -91,11 +91,13 @@ typedef struct {
   int max_levels;   /* 0 = planner default; otherwise the most qubit levels fused
                        into one pass (1..6), for tuning */
   int variant;      /* kernel form, for tuning: 0 = default (a single complex128
-                       matrix without zero skipping or partial masks runs the
-                       block fixed point's first pass, and the 2^11-element
-                       last pass of n = 15, as persistent CTAs, two per SM,
-                       each copying its next tile into shared memory while it
-                       finishes the current one), 1 = one CTA per tile
+                       matrix without zero skipping or partial masks runs a
+                       six-level first pass of the block fixed point as
+                       persistent CTAs, two per SM, each copying its next tile
+                       into shared memory while it finishes the current one,
+                       and the 2^12-element tiles of shorter first passes and
+                       of last passes, also in batched calls, as two halves, a
+                       CTA each), 1 = one CTA per tile
                        (complex128 tiles of 2^13 elements otherwise run as a
                        cluster of two 256-thread CTAs sharing the tile through
                        distributed shared memory),
@@ -484,8 +486,9 @@ void tpd_tune_clear(void);
 
 /* Describe the pass plan the library uses for (n, dtype, opt) as a
  * NUL-terminated text (one line per pass: levels, tile bits, tile count, the
- * CTAs per SM its kernel is compiled for, stages) written to buf (at most len
- * bytes).  Host only, no device call.  Returns the number
+ * CTAs per SM its kernel is compiled for, stages; where a pass's tiles run as
+ * two halves, a line "split pass ..." with the halves') written to buf (at most
+ * len bytes).  Host only, no device call.  Returns the number
  * of passes, or -1 on invalid arguments. */
 int tpd_plan_describe(int n, int dtype, const tpd_options* opt, char* buf, size_t len);
 

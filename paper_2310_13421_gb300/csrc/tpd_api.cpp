@@ -240,8 +240,16 @@ tpd_status run_single(bool dec, int arith, const void* src, void* mat, const Pla
   double sres = 1.0;
   if (!dec) split_scale(scale, &spow, &sres);
   const int variant = opt ? opt->variant : 0;
+  // L2 chunking: the first F passes run chunk by chunk, each chunk (the
+  // elements that agree on the global bits outside all F passes' tiles) small
+  // enough to stay in L2 from one pass to the next.
+  const L2Chunks ch = l2_chunks(plan, opt, skip || need || variant == 2);
+  // whole passes in the default form (or with their layouts read at run time)
+  // run split tiles as their halves
+  const bool halves = plan.split && !skip && !need && (variant == 0 || variant == 5) && ch.F < 2;
+  const PassDesc* const desc = halves ? plan.run : plan.pass;
   auto pass_args = [&](int p) {
-    const PassDesc& pd = plan.pass[p];
+    const PassDesc& pd = desc[p];
     const bool last = p + 1 == plan.npass;
     PassArgs a;
     std::memset(&a, 0, sizeof(a));
@@ -259,22 +267,18 @@ tpd_status run_single(bool dec, int arith, const void* src, void* mat, const Pla
     return a;
   };
   auto tuned_desc = [&](int p) {
-    PassDesc tuned = plan.pass[p];            // occupancy override (variants 3 and 4)
+    PassDesc tuned = desc[p];                 // occupancy override (variants 3 and 4)
     if (tuned.D <= 12 && (variant == 3 || variant == 4)) tuned.min_blocks = variant == 3 ? kOccLow : kOccHigh;
     if (tuned.D > 12 && variant == 1) tuned.min_blocks = 1;   // one 512-thread CTA per tile
     if (variant == 5) tuned.rt_layout = 1;    // layout read at run time
     return tuned;
   };
-  // L2 chunking: the first F passes run chunk by chunk, each chunk (the
-  // elements that agree on the global bits outside all F passes' tiles) small
-  // enough to stay in L2 from one pass to the next.
-  const L2Chunks ch = l2_chunks(plan, opt, skip || need || variant == 2);
   int p0 = 0;
   if (ch.F >= 2) {
     const int nfix = (int)ch.fixed.size();
     for (unsigned long long c = 0; c < (1ull << nfix); ++c)
       for (int p = 0; p < ch.F; ++p) {
-        const PassDesc& pd = plan.pass[p];
+        const PassDesc& pd = desc[p];
         PassArgs a = pass_args(p);
         a.chunked = 1;
         a.chunk_or = 0;
@@ -291,7 +295,7 @@ tpd_status run_single(bool dec, int arith, const void* src, void* mat, const Pla
     p0 = ch.F;
   }
   for (int p = p0; p < plan.npass; ++p) {
-    const PassDesc& pd = plan.pass[p];
+    const PassDesc& pd = desc[p];
     const PassArgs a = pass_args(p);
     const bool pipe = arith == kArithFixed && !skip && !need && pd.D <= 12 && variant == 2;
     const PassDesc tuned = tuned_desc(p);

@@ -232,8 +232,10 @@ tpd_status batched(bool dec, void* const* ptrs_dev, const int* ns_dev, const int
       size_t qoff = 0;
       const int16_t* q_prev = nullptr;
       long long q_prev_stride = 0;
+      const bool halves = plan.split && (variants[n] == 0 || variants[n] == 5);   // split tiles as their halves
+      const PassDesc* const desc = halves ? plan.run : plan.pass;
       for (int p = 0; p < plan.npass; ++p) {
-        const PassDesc& pd = plan.pass[p];
+        const PassDesc& pd = desc[p];
         const bool last = p + 1 == plan.npass;
         PassArgs a;
         std::memset(&a, 0, sizeof(a));

@@ -63,19 +63,36 @@ struct FixedArith {
   // x * 2^S truncated toward zero, S = 1084 - K - Emax_eff (see from_double).
   // shift_base = 9 - K - Emax_eff, so that the element with the tile's
   // largest exponent lands below 2^(62-K) and 2^K of them sum below 2^62.
+  // The mantissa is aligned to bit 63 (the funnel shift drops sign and
+  // exponent) and shifted down; PTX clamps shift amounts above 64 to 64
+  // (result 0): no undefined shifts.  The sign is a predicated negation.
   __device__ static __forceinline__ long long to_fixed(double x, int shift_base) {
-    const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
-    const int e = (int)(bits >> 52) & 0x7FF;
-    const unsigned long long m =
-        (bits & 0x000FFFFFFFFFFFFFull) | ((unsigned long long)(e != 0) << 52);
-    const int sh = max(e, 1) + shift_base;   // <= 9 - K <= 8
-    const unsigned rs = (unsigned)(11 - sh); // >= 3
-    unsigned long long mag;
-    const unsigned long long ml = m << 11;   // m < 2^53
-    // PTX clamps shift amounts above 64 to 64 (result 0): no undefined shifts.
-    asm("shr.b64 %0, %1, %2;" : "=l"(mag) : "l"(ml), "r"(rs));
-    const unsigned long long s = (unsigned long long)((long long)bits >> 63);
-    return (long long)((mag ^ s) - s);
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const int e = (int)(hi >> 20) & 0x7FF;
+    return shifted(hi, lo, e != 0 ? 0x80000000u : 0u, 11 - (max(e, 1) + shift_base));
+  }
+
+  // to_fixed for a class whose largest exponent field is at least kBigClass
+  // (shift_base <= 9 - K - kBigClass): an element without the implicit bit
+  // (zero or subnormal) is shifted out whether or not the bit is there.
+  static constexpr int kBigClass = 80;
+  __device__ static __forceinline__ long long to_fixed_big(double x, int shift_base) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    return shifted(hi, lo, 0x80000000u, 11 - ((int)((hi >> 20) & 0x7FFu) + shift_base));
+  }
+
+  // (implicit bit : mantissa) aligned to bit 63, shifted right by rs >= 3, with the sign of hi
+  __device__ static __forceinline__ long long shifted(uint32_t hi, uint32_t lo, uint32_t implicit, int rs) {
+    const uint32_t top = __funnelshift_l(lo, hi, 11) | implicit;
+    long long mag;
+    asm("{\n\t.reg .pred neg;\n\t.reg .b64 m;\n\t"
+        "mov.b64 m, {%1, %2};\n\t"
+        "shr.b64 %0, m, %3;\n\t"
+        "setp.lt.s32 neg, %4, 0;\n\t"
+        "@neg neg.s64 %0, %0;\n\t}"
+        : "=&l"(mag)
+        : "r"(lo << 11), "r"(top), "r"(rs), "r"((int)hi));
+    return mag;
   }
 
   // The same value through the fp64 conversion unit: scale by 2^S with an

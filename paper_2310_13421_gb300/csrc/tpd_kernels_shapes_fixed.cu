@@ -18,6 +18,8 @@ PassKernel fixed_table(int shape, int role) {
     case kShapeFirst6 * 4 + kOut: return fixed_k<kDec, kMin, kOut, kShapeFirst6>();
     case kShapeFirst5 * 4 + kOut: return fixed_k<kDec, kMin, kOut, kShapeFirst5>();
     case kShapeFirst4 * 4 + kOut: return fixed_k<kDec, kMin, kOut, kShapeFirst4>();
+    case kShapeFirst5D11 * 4 + kOut: return fixed_k<kDec, kMin, kOut, kShapeFirst5D11>();
+    case kShapeFirst4D11 * 4 + kOut: return fixed_k<kDec, kMin, kOut, kShapeFirst4D11>();
     case kShapeMid4 * 4 + kInOut: return fixed_k<kDec, kMin, kInOut, kShapeMid4>();
     case kShapeMid4 * 4 + kIn: return fixed_k<kDec, kMin, kIn, kShapeMid4>();
     case kShapeMid4D11 * 4 + kIn: return fixed_k<kDec, kMin, kIn, kShapeMid4D11>();
@@ -34,19 +36,12 @@ PassKernel shape_kernel_fixed(bool dec, int shape, int role, int min_blocks) {
 
 // The persistent prefetching form (k_pass_pf) of the decomposition for a
 // compiled layout and role where it was measured faster on GB300, or nullptr:
-// the first passes (double -> int64; n = 14 first pass 1.864 -> 1.754 ms,
-// n = 15 7.50 -> 6.97 ms) and the last pass of n = 15 on 2^11-element tiles
-// (7.72 -> 7.12 ms); the later passes on 2^12-element tiles ran as fast or
-// slower (n = 14 last pass 1.703 -> 1.870 ms).
+// the six-level first pass on 2^12-element tiles (n = 14 1.864 -> 1.754 ms).
+// Two CTAs per SM need it; four of 128 threads on 2^11 elements overlap each
+// other better (n = 13 first pass 0.395 with it, 0.346 ms without; n = 15 last
+// pass 6.52, 6.34 ms; n = 14 middle pass 1.49, 1.43 ms).
 PassKernel shape_kernel_fixed_pf(int shape, int role) {
-  constexpr int kIn = kRoleIntIn, kOut = kRoleIntOut;
-  switch (shape * 4 + role) {
-    case kShapeFirst6 * 4 + kOut: return k_pass_pf<true, kOut, kShapeFirst6>;
-    case kShapeFirst5 * 4 + kOut: return k_pass_pf<true, kOut, kShapeFirst5>;
-    case kShapeFirst4 * 4 + kOut: return k_pass_pf<true, kOut, kShapeFirst4>;
-    case kShapeMid4D11 * 4 + kIn: return k_pass_pf<true, kIn, kShapeMid4D11>;
-    default: return nullptr;
-  }
+  return shape == kShapeFirst6 && role == kRoleIntOut ? k_pass_pf<true, kRoleIntOut, kShapeFirst6> : nullptr;
 }
 
 // 2^13-element tiles as two-CTA clusters (the 5-level passes of n = 11 and 15)

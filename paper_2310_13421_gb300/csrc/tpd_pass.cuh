@@ -567,33 +567,31 @@ __device__ __forceinline__ void class_atomics_any(int np, const T (&x)[kElems], 
   else class_atomics<0, S>(x, slots, ct, c0, c1, c2, c3);
 }
 
-// Returns the largest exponent field of the thread's elements, and in lo
-// the smallest nonzero one (0x7fffffff if none).
-template <class S, class G, class Raw, class ExpOf>
-__device__ __forceinline__ uint32_t class_max(const G& pd, const Raw (&raw)[kElems], int* slots, int lane,
-                                              int warp, ExpOf exp_of, int& lo) {
+// Class maxima of a loaded tile's exponent fields (see class_atomics).
+template <class S, class G, class Raw>
+__device__ __forceinline__ void class_max(const G& pd, const Raw (&raw)[kElems], int* slots, int lane, int warp) {
   const auto& s0 = pd.st[0];
   const int ct = cls_thread(pd, s0, lane, warp);
   const int c0 = pd.cls_w[s0.reg[0]], c1 = pd.cls_w[s0.reg[1]], c2 = pd.cls_w[s0.reg[2]],
             c3 = pd.cls_w[s0.reg[3]];
-  uint32_t hmax = 0, hmin = 0x7fffffffu;
-#pragma unroll
-  for (int e = 0; e < kElems; ++e) {
-    const uint32_t x = exp_of(raw[e]);
-    hmax = max(hmax, x);
-    hmin = min(hmin, x ? x : 0x7fffffffu);
-  }
-  lo = (int)hmin;
-  // (the exponents are recomputed rather than kept: 16 registers fewer)
   class_atomics_any<S>(s0.npair, raw, slots, ct, c0, c1, c2, c3);
-  return hmax;
 }
 
-__device__ __forceinline__ uint32_t exp_f64(const double2& x) {
-  return max((uint32_t)__double2hiint(x.x) & 0x7fffffffu, (uint32_t)__double2hiint(x.y) & 0x7fffffffu) >> 20;
-}
-__device__ __forceinline__ uint32_t exp_f32(const float2& x) {
-  return max(__float_as_uint(x.x) & 0x7fffffffu, __float_as_uint(x.y) & 0x7fffffffu) >> 23;
+// Range of the nonzero class slots (lo = 0x7fffffff, hi = 0: none) and whether
+// any is 0, once they are complete: every warp reads them all, so that nothing
+// more is exchanged.
+__device__ __forceinline__ void slot_range(const int* cls, int ncls, int lane, int& lo, int& hi, bool& zero) {
+  uint32_t l = 0x7fffffffu, h = 0;
+  bool z = false;
+  for (int i = lane; i < ncls; i += 32) {
+    const uint32_t x = (uint32_t)cls[i];
+    z |= x == 0;
+    h = max(h, x);
+    l = min(l, x ? x : 0x7fffffffu);
+  }
+  lo = (int)__reduce_min_sync(kFull, l);
+  hi = (int)__reduce_max_sync(kFull, h);
+  zero = __any_sync(kFull, z);
 }
 
 // Source-class index (previous pass's binary-point array) of a thread's
@@ -626,10 +624,17 @@ __device__ __forceinline__ long long shr_floor(long long v, unsigned sh) {
 // v / 2^sh rounded toward zero (sh >= 0; 0 once sh >= 64): an odd function,
 // so conjugate sums stay exactly conjugate
 __device__ __forceinline__ long long shr_tz(long long v, unsigned sh) {
-  const unsigned long long s = (unsigned long long)(v >> 63);
-  unsigned long long a = ((unsigned long long)v ^ s) - s;
-  asm("shr.b64 %0, %0, %1;" : "+l"(a) : "r"(sh));   // PTX clamps the amount at 64
-  return (long long)((a ^ s) - s);
+  // the magnitude shifted between two negations predicated on the high word's
+  // sign (n = 14 middle pass 1.405 ms; predicated on the 64-bit value 1.432,
+  // by xor and subtract 1.416, by a floor shift and a correction 1.422)
+  long long r = v;
+  asm("{\n\t.reg .pred neg;\n\t"
+      "setp.lt.s32 neg, %1, 0;\n\t"
+      "@neg neg.s64 %0, %0;\n\t"
+      "shr.u64 %0, %0, %2;\n\t"                      // PTX clamps the amount at 64
+      "@neg neg.s64 %0, %0;\n\t}"
+      : "+l"(r) : "r"((int)(v >> 32)), "r"(sh));
+  return r;
 }
 
 // Tiles meeting an Inf or NaN run the IEEE fp64 butterfly instead (rounded
@@ -701,30 +706,49 @@ __device__ __forceinline__ void flag_next(const G& pd, const PassArgs& args, int
   }
 }
 
-// Tile-wide reduction of the flags (OR) and of the range [lo, hi] of the
-// nonzero class slots, through red[0..S) / red[S..2S) / red[2S..3S), S = kRedStride (one
-// entry per warp; a two-CTA cluster writes its entries into both CTAs at the
-// one-CTA layout's warp index and meets at a cluster barrier).
+// Tile-wide barrier with the OR of a flag (a two-CTA cluster writes one entry
+// per warp into both CTAs' red[] at the one-CTA layout's warp index and meets
+// at a cluster barrier).
 template <bool kCl>
-__device__ __forceinline__ void tile_reduce(int* red, int warp, int lane, int nwarps_total, int& tb, int& lo,
-                                            int& hi) {
-  tb = __reduce_or_sync(kFull, tb);
-  lo = (int)__reduce_min_sync(kFull, (unsigned)lo);
-  hi = (int)__reduce_max_sync(kFull, (unsigned)hi);
-  if (lane == 0) {
-    red[warp] = tb; red[kRedStride + warp] = lo; red[2 * kRedStride + warp] = hi;
-    if constexpr (kCl) {
-      int* pr = peer_smem(red);
-      pr[warp] = tb; pr[kRedStride + warp] = lo; pr[2 * kRedStride + warp] = hi;
+__device__ __forceinline__ int tile_or(int flag, int* red, int warp, int lane, int nwarps_total) {
+  if constexpr (kCl) {
+    flag = __any_sync(kFull, flag) ? 1 : 0;
+    if (lane == 0) {
+      red[warp] = flag;
+      peer_smem(red)[warp] = flag;
     }
+    cluster_sync();
+    return __any_sync(kFull, lane < nwarps_total && red[lane < nwarps_total ? lane : 0] != 0) ? 1 : 0;
+  } else {
+    return __syncthreads_or(flag);
   }
+}
+template <bool kCl>
+__device__ __forceinline__ void tile_sync() {
   if constexpr (kCl) cluster_sync();
   else __syncthreads();
-  // lane w reads warp w's entries; one warp-wide reduction each
-  const bool in = lane < nwarps_total;
-  tb = (int)__reduce_or_sync(kFull, in ? (unsigned)red[lane] : 0u);
-  lo = (int)__reduce_min_sync(kFull, in ? (unsigned)red[kRedStride + lane] : 0x7fffffffu);
-  hi = (int)__reduce_max_sync(kFull, in ? (unsigned)red[2 * kRedStride + lane] : 0u);
+}
+// both CTAs' class slots of a cluster, merged (after a tile barrier)
+template <bool kCl>
+__device__ __forceinline__ void merge_slots(int* cls, int ncls, int nthr) {
+  if constexpr (kCl) {
+    const int* pcls = peer_smem(cls);
+    int mine[8];                                         // 2^(D-K) slots over 256 threads: at most 16 for K = 1
+    for (int i0 = 0; i0 < ncls; i0 += 8 * nthr) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int i = i0 + k * nthr + (int)threadIdx.x;
+        mine[k] = i < ncls ? max(cls[i], pcls[i]) : 0;
+      }
+      cluster_sync();                                    // both CTAs have read these
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int i = i0 + k * nthr + (int)threadIdx.x;
+        if (i < ncls) cls[i] = mine[k];
+      }
+    }
+    __syncthreads();
+  }
 }
 
 // Asynchronous copies of a tile's elements into shared memory (the
@@ -799,13 +823,13 @@ __device__ __forceinline__ void fixed_tile(const G& pd, const PassArgs& args, vo
   const int ncls = 1 << (pd.D - pd.K);
   for (int i = threadIdx.x; i < ncls; i += nthr) cls[i] = 0;
   int slot_lo, slot_hi;                                  // range of the tile's nonzero class slots
+  bool zero_slot;                                        // a class without a normal number
   const auto& s0 = pd.st[0];
   const int ct = cls_thread(pd, s0, lane, warp);
   const int c0 = pd.cls_w[s0.reg[0]], c1 = pd.cls_w[s0.reg[1]], c2 = pd.cls_w[s0.reg[2]],
             c3 = pd.cls_w[s0.reg[3]];
   const int np = s0.npair;
   V v[kElems];
-  int tb;                                                // tile flags: 1 nonzero, 2 Inf / NaN
   if constexpr (!kIntIn) {
     // ---- IEEE doubles: class maxima of the exponent fields
     double2 raw[kElems];
@@ -813,22 +837,22 @@ __device__ __forceinline__ void fixed_tile(const G& pd, const PassArgs& args, vo
     else load_tile<kCg>(pd, pass_input<kRole>(args, matp), base, lane, warp, raw);
     if constexpr (kCl) cluster_wait();                   // the peer CTA is running
     __syncthreads();                                     // class slots cleared
-    int lo;
-    const uint32_t hmax = class_max<ExpSlot64>(pd, raw, cls, lane, warp, exp_f64, lo);
-    uint32_t nzw = 0;
+    class_max<ExpSlot64>(pd, raw, cls, lane, warp);
+    bool zero = false;
     if (args.skip_zero) {
+      uint32_t nzw = 0;
 #pragma unroll
       for (int e = 0; e < kElems; ++e)
         nzw |= (uint32_t)__double2hiint(raw[e].x) << 1 | (uint32_t)__double2loint(raw[e].x) |
                (uint32_t)__double2hiint(raw[e].y) << 1 | (uint32_t)__double2loint(raw[e].y);
+      zero = !tile_or<kCl>(nzw != 0, red, warp, lane, nwarps_total);
+    } else {
+      tile_sync<kCl>();                                  // both CTAs' atomics are in
     }
-    tb = (nzw != 0 ? 1 : 0) | (hmax == 2047 ? 2 : 0);
-    int hi = (int)hmax;
-    tile_reduce<kCl>(red, warp, lane, nwarps_total, tb, lo, hi);   // both CTAs' atomics and flags are in
-    slot_lo = lo;
-    slot_hi = hi;
-    if ((args.skip_zero && !(tb & 1)) || (tb & 2)) {
-      if (tb & 2)
+    merge_slots<kCl>(cls, ncls, nthr);
+    slot_range(cls, ncls, lane, slot_lo, slot_hi, zero_slot);
+    if (zero || slot_hi == 2047) {
+      if (slot_hi == 2047)                               // Inf / NaN
         ieee_tile<kDec, kCg, kCl>(raw_desc(pd), args, matp, q_in, q_out, tile, base, sbase, nbase, xbuf, lane,
                                   warp);
       else if (args.src != nullptr)
@@ -836,17 +860,21 @@ __device__ __forceinline__ void fixed_tile(const G& pd, const PassArgs& args, vo
       prefetch_next();
       return;                                            // (else all +-0: the outputs are zero already)
     }
-    if constexpr (kCl) {
-      const int* pcls = peer_smem(cls);
-      for (int i = threadIdx.x; i < ncls; i += nthr) cls[i] = max(cls[i], pcls[i]);
-      cluster_sync();                                    // both CTAs are done with the peer's slots
-    }
     // onto the classes' binary points: x * 2^S_c, S_c = 1084 - K - max(E_c, 1)
+    if (!zero_slot && slot_lo >= FixedArith::kBigClass) {  // dense data
 #pragma unroll
-    for (int e = 0; e < kElems; ++e) {
-      const int sb = 9 - pd.K - max(cls[ct ^ reg_cls(e, c0, c1, c2, c3)], 1);
-      v[e].re = FixedArith::to_fixed(raw[e].x, sb);
-      v[e].im = FixedArith::to_fixed(raw[e].y, sb);
+      for (int e = 0; e < kElems; ++e) {
+        const int sb = 9 - pd.K - cls[ct ^ reg_cls(e, c0, c1, c2, c3)];
+        v[e].re = FixedArith::to_fixed_big(raw[e].x, sb);
+        v[e].im = FixedArith::to_fixed_big(raw[e].y, sb);
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < kElems; ++e) {
+        const int sb = 9 - pd.K - max(cls[ct ^ reg_cls(e, c0, c1, c2, c3)], 1);
+        v[e].re = FixedArith::to_fixed(raw[e].x, sb);
+        v[e].im = FixedArith::to_fixed(raw[e].y, sb);
+      }
     }
   } else {
     // ---- int64 sums of a previous pass, each with its source class's binary point
@@ -863,34 +891,22 @@ __device__ __forceinline__ void fixed_tile(const G& pd, const PassArgs& args, vo
     }
     if constexpr (kCl) cluster_wait();                   // the peer CTA is running
     __syncthreads();                                     // class slots cleared
-    int any_valid = 0, any_ieee = 0, lo = 0x7fffffff, hi = 0;
+    int any_ieee = 0;
 #pragma unroll
-    for (int e = 0; e < kElems; ++e) {
-      const bool ok = q_is_valid(qs[e]);
-      any_valid |= ok;
-      any_ieee |= qs[e] == kQIeee;
-      lo = min(lo, ok ? qs[e] + kQSlot : 0x7fffffff);
-      hi = max(hi, ok ? qs[e] + kQSlot : 0);
-    }
+    for (int e = 0; e < kElems; ++e) any_ieee |= qs[e] == kQIeee;
     class_atomics_any<QSlot>(np, qs, cls, ct, c0, c1, c2, c3);
-    tb = (any_valid ? 1 : 0) | (any_ieee ? 2 : 0);
-    tile_reduce<kCl>(red, warp, lane, nwarps_total, tb, lo, hi);
-    slot_lo = lo;
-    slot_hi = hi;
-    if (tb & 2) {
+    any_ieee = tile_or<kCl>(any_ieee, red, warp, lane, nwarps_total);
+    if (any_ieee) {
       ieee_tile<kDec, kCg, kCl>(raw_desc(pd), args, matp, q_in, q_out, tile, base, sbase, nbase, xbuf, lane,
                                 warp);
       prefetch_next();
       return;
     }
-    if (args.skip_zero && !(tb & 1)) {                   // every source class was zero
+    merge_slots<kCl>(cls, ncls, nthr);
+    slot_range(cls, ncls, lane, slot_lo, slot_hi, zero_slot);
+    if (args.skip_zero && slot_hi == 0) {                // every source class was zero
       prefetch_next();
       return;
-    }
-    if constexpr (kCl) {
-      const int* pcls = peer_smem(cls);
-      for (int i = threadIdx.x; i < ncls; i += nthr) cls[i] = max(cls[i], pcls[i]);
-      cluster_sync();
     }
     // realign onto q_in_c = (largest source point) + K.  Conjugate partners
     // (Hermitian inputs) have equal real parts and opposite imaginary parts:
@@ -956,7 +972,22 @@ __device__ __forceinline__ void fixed_tile(const G& pd, const PassArgs& args, vo
     const int tadj = -(kDec ? pd.K : 0) + args.out_pow2;
     const bool fast = !resid && (slot_hi < slot_lo || (FixedArith::fast_range(-(q_of_slot(slot_hi) + tadj)) &&
                                                        FixedArith::fast_range(-(q_of_slot(slot_lo) + tadj))));
-    if (fast) {
+    // a Hermitian matrix's weights are real, exactly: where a warp's imaginary
+    // sums are all 0 they need no conversion (n = 14 last pass 1.74 -> 1.58 ms)
+    bool real = false;
+    if constexpr (kDec) {
+      long long im = 0;
+#pragma unroll
+      for (int e = 0; e < kElems; ++e) im |= v[e].im;
+      real = __all_sync(kFull, im == 0);
+    }
+    if (fast && real) {
+#pragma unroll
+      for (int e = 0; e < kElems; ++e) {
+        const int T = -(q_of_slot(cls[cl ^ reg_cls(e, l0, l1, l2, l3)]) + tadj);
+        mat[g + reg_off(e, w0, w1, w2, w3)] = make_double2(FixedArith::to_double_cvt_fast(v[e].re, T), 0.0);
+      }
+    } else if (fast) {
       // real parts through the fp64 conversion unit, imaginary parts through
       // integer instructions (identical roundings): the two pipes share the
       // conversions
@@ -984,25 +1015,27 @@ __device__ __forceinline__ void fixed_tile(const G& pd, const PassArgs& args, vo
 // float butterfly instead.
 template <bool kDec, bool kCg, class G>
 __device__ __forceinline__ void fixed32_tile(const G& pd, const PassArgs& args, void* matp, long long base,
-                                             int nbase, unsigned char* smem, int* red, int* cls, int lane, int warp) {
+                                             int nbase, unsigned char* smem, int* cls, int lane, int warp) {
   using V = Fixed32Arith::V;
-  const int nthr = blockDim.x, nwarps = nthr >> 5;
+  const int nthr = blockDim.x;
   const int ncls = 1 << (pd.D - pd.K);
   for (int i = threadIdx.x; i < ncls; i += nthr) cls[i] = 0;
   float2 raw[kElems];
   load_tile<kCg>(pd, pass_input<0>(args, matp), base, lane, warp, raw);
   __syncthreads();                                       // class slots cleared
-  int lo_unused;
-  const uint32_t hmax = class_max<ExpSlot32>(pd, raw, cls, lane, warp, exp_f32, lo_unused);
+  class_max<ExpSlot32>(pd, raw, cls, lane, warp);
   uint32_t nzw = 0;
   if (args.skip_zero) {
 #pragma unroll
     for (int e = 0; e < kElems; ++e) nzw |= (__float_as_uint(raw[e].x) | __float_as_uint(raw[e].y)) << 1;
+    if (!__syncthreads_or(nzw != 0)) return;             // all +-0: the outputs are zero already
+  } else {
+    __syncthreads();
   }
-  int t = (nzw != 0 ? 1 : 0) | (hmax == 255 ? 2 : 0), hi_unused = 0;
-  tile_reduce<false>(red, warp, lane, nwarps, t, lo_unused, hi_unused);
-  if (args.skip_zero && !(t & 1)) return;                // all +-0: the outputs are zero already
-  if (t & 2) {                                           // Inf/NaN in the tile
+  int slot_lo, slot_hi;
+  bool zero_slot;
+  slot_range(cls, ncls, lane, slot_lo, slot_hi, zero_slot);
+  if (slot_hi == 255) {                                  // Inf/NaN in the tile
     finish_tile<F32Arith, kDec>(pd, args, matp, raw, kDec ? pow2d(-pd.K) : pow2d(args.out_pow2) * args.out_mul,
                                 base, nbase, smem, lane, warp);
     return;
@@ -1078,7 +1111,7 @@ __device__ __forceinline__ void pass_tile(const G& pd, const PassArgs& args, voi
     fixed_tile<kDec, kRole, kCg, kCl>(pd, args, matp, q_in, q_out, tile, base, sbase, nbase, nullptr, smem,
                                       red, cls, lane, warp);
   } else if constexpr (A::kFixed32) {
-    fixed32_tile<kDec, kCg>(pd, args, matp, base, nbase, smem, red, cls, lane, warp);
+    fixed32_tile<kDec, kCg>(pd, args, matp, base, nbase, smem, cls, lane, warp);
   } else {
     Store raw[kElems];
     load_tile<kCg>(pd, pass_input<0>(args, matp), base, lane, warp, raw);
@@ -1359,7 +1392,7 @@ __device__ __forceinline__ void small_matrix(const typename A::Store* src, typen
     uint32_t hmax = 0, nzw = 0;
     for (int i = tid; i < count; i += nthr) {
       const double2 x = src[i];
-      const uint32_t ex = exp_f64(x);
+      const uint32_t ex = (uint32_t)ExpSlot64::of(x);
       hmax = max(hmax, ex);
       nzw |= (uint32_t)__double2hiint(x.x) << 1 | (uint32_t)__double2loint(x.x) |
              (uint32_t)__double2hiint(x.y) << 1 | (uint32_t)__double2loint(x.y);

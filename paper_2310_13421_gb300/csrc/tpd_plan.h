@@ -116,6 +116,12 @@ struct Plan {
   int32_t npass;
   int32_t elem_bytes;        // 16 (c128, compensated c64 in registers) or 8
   PassDesc pass[kMaxQubits];  // one level per pass at worst
+  // Split tiles (bit p of split: pass p): the descriptors of a run in which
+  // those passes' tiles are halved (valid if split != 0, every pass's: the
+  // binary points a pass hands on are indexed by its tiles, so the next one's
+  // src_w depends on them).  As many classes, so the same workspace.
+  uint32_t split;
+  PassDesc run[kMaxQubits];
 };
 
 }  // namespace tpd

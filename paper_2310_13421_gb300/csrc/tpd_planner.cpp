@@ -308,8 +308,9 @@ bool build_plan(int n, int dtype, int precision, int tile_bits_opt, int max_leve
     // 128 threads per SM instead of two of 256) -- measured on GB300 with the
     // compiled layouts, n = 14 middle pass 1.550 -> 1.397 ms, n = 13 0.374 ->
     // 0.340 ms, n = 16 25.9 / 26.9 -> 21.5 / 24.7 ms; the first and last
-    // passes keep 2^12 (the last one ran 3-4 % slower on 2^11), complex64
-    // keeps 2^12 (plain n = 14 passes 0.62 / 0.64 -> 0.68 / 0.74 ms)
+    // passes are planned on 2^12 (see the split tiles below), complex64
+    // keeps 2^12 (plain n = 14 passes 0.62 / 0.64 -> 0.68 / 0.74 ms;
+    // compensated n = 15 first 3.15 -> 3.27, last 2.98 -> 3.26 ms)
     if (dtype == 0 && !tile_bits_opt)
       for (size_t i = 1; i + 1 < g.size(); ++i) {
         const int Dsmall = std::max(kMinTileBits, 2 * g[i].first + lf);
@@ -387,6 +388,32 @@ bool build_plan(int n, int dtype, int precision, int tile_bits_opt, int max_leve
     pd.shape = match_shape(pd);
     pd.min_blocks = pd.D > 12 ? (dtype == 0 ? 2 : 1) : (three ? kOccHigh : kOccLow);
   }
+  // Split tiles: a first pass of up to 5 levels or a last one of 4 in the
+  // complex128 block fixed point, planned on 2^12-element tiles, holds a
+  // passenger bit it does not need: its highest splits the tile into two
+  // independent halves, each run by a CTA of 128 threads of its own, four per
+  // SM instead of two of 256 that wait at the same barriers.  GB300: n = 13
+  // first pass 0.431 -> 0.346 ms, n = 12 0.110 -> 0.095 ms (on quarters 0.340 /
+  // 0.094, but n = 9 0.0107 -> 0.0122 ms); n = 14 last pass 1.73 -> 1.58 ms,
+  // general matrices 1.88 -> 1.74 ms.  Six levels have no such bit.  Whole
+  // passes only (no zero skipping, masks or other variants), and where the
+  // half's layout is compiled.
+  if (dtype == 0 && precision == 3 && !tile_bits_opt && plan->npass > 1) {
+    for (int p = 0; p < plan->npass; ++p) {
+      const PassDesc& pd = plan->pass[p];
+      PassDesc& h = plan->run[p];
+      h = pd;
+      if (pd.D != 12 || 2 * pd.K + (p > 0 ? lf : 0) > 11) continue;
+      PassDesc half;
+      if (!build_pass(n, pd.b, pd.K, 11, lf, cs, &half, err)) return false;
+      half.shape = match_shape(half);
+      half.min_blocks = kOccLow;
+      if (half.shape < 0) continue;
+      h = half;
+      plan->split |= 1u << p;
+    }
+    for (int p = 1; p < plan->npass; ++p) set_src(&plan->run[p], plan->run[p - 1]);
+  }
   return true;
 }
 
@@ -398,9 +425,12 @@ std::string describe_plan(const Plan& plan) {
                   1 << (2 * plan.n));
     return buf;
   }
-  for (int p = 0; p < plan.npass; ++p) {
-    const PassDesc& pd = plan.pass[p];
-    std::snprintf(buf, sizeof(buf), "pass %d: levels [%d,%d) D=%d tiles=%lld ctas=%d gbits=", p, pd.b,
+  // a pass whose tiles run split has a second line, "split pass ...": the halves
+  for (int q = 0; q < 2 * plan.npass; ++q) {
+    const int p = q / 2;
+    if ((q & 1) && !((plan.split >> p) & 1u)) continue;
+    const PassDesc& pd = (q & 1) ? plan.run[p] : plan.pass[p];
+    std::snprintf(buf, sizeof(buf), "%spass %d: levels [%d,%d) D=%d tiles=%lld ctas=%d gbits=", (q & 1) ? "split " : "", p, pd.b,
                   pd.b + pd.K, pd.D, (long long)pd.ntiles, pd.min_blocks);
     s += buf;
     for (int i = 0; i < pd.D; ++i) {

@@ -42,9 +42,11 @@ enum ShapeId {
   kShapeFirst5,       // 5 levels on 2^12 (n = 13 and others)
   kShapeMid4,         // 4 levels + 4 passengers on 2^12 (most later passes)
   kShapeFirst4,       // 4 levels on 2^12, complex64 compensated first pass (128-byte runs)
-  kShapeMid4D11,      // 4 levels + 3 passengers on 2^11 (complex128 middle passes, n = 15 last pass)
+  kShapeMid4D11,      // 4 levels + 3 passengers on 2^11 (complex128 later passes)
   kShapeMid3,         // 3 levels + 6 passengers on 2^12 (compensated complex64 last passes)
   kShapeMid5D13,      // 5 levels + 3 passengers on 2^13, one 512-thread CTA (complex64 n = 11, 15)
+  kShapeFirst5D11,    // 5 levels on 2^11 (complex128 first passes: n = 13, 9, 7)
+  kShapeFirst4D11,    // 4 levels on 2^11 (complex128 first passes: n = 12, 16)
   kNumShapes
 };
 
@@ -112,6 +114,24 @@ constexpr ShapeDesc kShapes[kNumShapes] = {
      {2, 0, 0},
      {{3, 4, 0, 0}, {0, 0, 0, 0}, {0, 0, 0, 0}},
      {0, 1, 2, 3, 4, 5, 6, 7, 3, 4, 5, 6, 7}},
+    // kShapeFirst5D11: levels 0-4 + 1 passenger
+    {11, 5, 2,
+     {{6, 7, 8, 10}, {3, 9, 4, 10}, {0, 0, 0, 0}},
+     {{0, 1, 2, 3, 4}, {0, 1, 2, 5, 6}, {0, 0, 0, 0, 0}},
+     {{5, 9, 0, 0}, {7, 8, 0, 0}, {0, 0, 0, 0}},
+     {0, 2, 0},
+     {3, 0, 0},
+     {{0, 1, 2, 0}, {0, 0, 0, 0}, {0, 0, 0, 0}},
+     {0, 1, 2, 3, 4, 5, 0, 1, 2, 3, 4, 0, 0}},
+    // kShapeFirst4D11: levels 0-3 + 3 passengers, one stage of four shuffle levels
+    {11, 4, 1,
+     {{7, 8, 9, 10}, {0, 0, 0, 0}, {0, 0, 0, 0}},
+     {{0, 1, 2, 3, 4}, {0, 0, 0, 0, 0}, {0, 0, 0, 0, 0}},
+     {{5, 6, 0, 0}, {0, 0, 0, 0}, {0, 0, 0, 0}},
+     {0, 0, 0},
+     {4, 0, 0},
+     {{0, 1, 2, 3}, {0, 0, 0, 0}, {0, 0, 0, 0}},
+     {0, 1, 2, 3, 4, 5, 6, 0, 1, 2, 3, 0, 0}},
 };
 
 // Packed forms (4 bits per tile-bit number, 3 per shuffle lane) from which
