@@ -319,8 +319,8 @@ tpd_status tpd_nonzero_write(const void* W, int n, int dtype, double tol, unsign
  *   values      device, nnz complex128.
  *   n           1..15.
  *   max_entries the most entries any level may hold (device memory grows with
- *               it: about 52 bytes per entry); more sets *status to
- *               TPD_ERR_WORKSPACE and the list is incomplete.  A level holds
+ *               it: 112 to 192 bytes per entry); more sets *status to
+ *               TPD_ERR_WORKSPACE and the list is empty (*count = 0).  A level holds
  *               at most 2x the entries of the one before.
  *   strings, weights, capacity, count   as tpd_nonzero_list.
  *   status      device, one unsigned (may be NULL): TPD_OK or TPD_ERR_WORKSPACE.

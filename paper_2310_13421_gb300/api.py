@@ -284,18 +284,18 @@ def decompose_coo(rows, cols, values, n, *, max_entries=None, capacity=None, str
     cap_entries = int(max_entries) if max_entries else 4 * nnz + 1024
     while True:
         with _enqueue(dev, stream, rows, cols, values) as s:
-            count = torch.zeros(1, dtype=torch.int64, device=dev)
-            status = torch.zeros(1, dtype=torch.int32, device=dev)
+            meta = torch.zeros(2, dtype=torch.int64, device=dev)      # count, status: read back together
             ws = torch.empty(L.tpd_sparse_workspace_size(cap_entries), dtype=torch.uint8, device=dev)
             cap = int(capacity) if capacity is not None else cap_entries
             strings = torch.empty(max(cap, 1), dtype=torch.int64, device=dev)
             weights = torch.empty(max(cap, 1), dtype=torch.complex128, device=dev)
             st = L.tpd_decompose_coo(rows.data_ptr(), cols.data_ptr(), values.data_ptr(), nnz, int(n), L.TPD_C128,
-                                     cap_entries, strings.data_ptr(), weights.data_ptr(), cap, count.data_ptr(),
-                                     status.data_ptr(), ws.data_ptr(), ws.numel(), s)
-        _raise(st, "tpd_decompose_coo")
-        if int(status.item()) == 0:
-            k = min(int(count.item()), cap)
+                                     cap_entries, strings.data_ptr(), weights.data_ptr(), cap, meta.data_ptr(),
+                                     meta.data_ptr() + 8, ws.data_ptr(), ws.numel(), s)
+            _raise(st, "tpd_decompose_coo")
+            found, status = meta.tolist()                              # waits for this stream
+        if status == 0:
+            k = min(found, cap)
             return strings[:k], weights[:k]
         if max_entries:
             raise L.TPDError(L.TPD_ERR_WORKSPACE, "tpd_decompose_coo (max_entries too small)")

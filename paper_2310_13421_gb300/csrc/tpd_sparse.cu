@@ -12,7 +12,18 @@
 // the end as 2^-n):
 //     a00 -> I +v, Z +v     a11 -> I +v, Z -v
 //     a01 -> X +v, Y +iv    a10 -> X +v, Y -iv
-// Entries with equal keys are summed in a hash table, zero sums dropped.
+// Entries with equal keys are summed in a hash table, zero sums dropped: one
+// launch a level reads the table that the level before filled, drops its zero
+// sums, empties it and adds the others' children to a second table.  The
+// launches, not the entries, set the time of small problems, so the sort of
+// the final list is one launch per doubling beyond 2048 entries, and a
+// counter is touched once a CTA.  GB300, n = 14 Heisenberg chain (122,880
+// entries, 53 strings): 0.70 -> 0.29 ms a call with its synchronisation, against
+// an entry list between two launches a level (9 and 26 us), an atomic an entry on
+// its counter and a launch per bitonic step, 80 launches against 27.  A level
+// takes 5-11 us, round trips to L2 and little else: with the entries left in
+// their slots' lanes it took 70-90 us, and with the values loaded one after
+// another, at six CTAs an SM, 16-29 us.
 //
 // Exactness: values are int64 on one binary point per X-mask x = r xor c
 // (x * 2^S_x, S_x = 1084 - n - the largest exponent among the entries of that
@@ -50,7 +61,10 @@ __global__ void k_sp_emax(const int* __restrict__ rows, const int* __restrict__ 
     const int ex = (int)((unsigned long long)__double_as_longlong(vals[i].x) >> 52) & 0x7FF;
     const int ey = (int)((unsigned long long)__double_as_longlong(vals[i].y) >> 52) & 0x7FF;
     const int e = max(ex, ey);
-    if (e) atomicMax(emax + ((rows[i] ^ cols[i]) & xmask), e);
+    // read first: an X-mask's entries mostly share a magnitude, and atomics on
+    // one address (the diagonal's) serialise (26 -> 18 us for 122,880 entries)
+    int* const p = emax + ((rows[i] ^ cols[i]) & xmask);
+    if (e > *reinterpret_cast<const volatile int*>(p)) atomicMax(p, e);
   }
 }
 
@@ -96,26 +110,19 @@ __device__ __forceinline__ double sp_to_double(long long v, int T) {
   return __longlong_as_double((long long)(bits | (s & 0x8000000000000000ull)));
 }
 
-// initial entries: key = r*N + c, value on its X-mask's binary point
-__global__ void k_sp_init(const int* __restrict__ rows, const int* __restrict__ cols, const double2* __restrict__ vals,
-                          unsigned long long m, int n, const int* __restrict__ emax, uint32_t* __restrict__ keys,
-                          longlong2* __restrict__ v) {
-  const unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
-  if (i >= m) return;
-  const int emax_eff = max(emax[(rows[i] ^ cols[i]) & ((1 << n) - 1)], 1);
-  keys[i] = ((uint32_t)rows[i] << n) | (uint32_t)cols[i];
-  v[i] = make_longlong2(sp_to_fixed(vals[i].x, n, emax_eff), sp_to_fixed(vals[i].y, n, emax_eff));
+__device__ __forceinline__ void sp_add(unsigned long long* __restrict__ tv, uint32_t slot, long long re, long long im) {
+  atomicAdd(tv + 2ull * slot, (unsigned long long)re);         // two's complement: exact int64 sums
+  atomicAdd(tv + 2ull * slot + 1, (unsigned long long)im);
 }
 
-__device__ __forceinline__ void sp_insert(uint32_t key, long long re, long long im, uint32_t* __restrict__ tkeys,
-                                          unsigned long long* __restrict__ tv, uint32_t mask,
-                                          unsigned long long* __restrict__ overflow) {
-  uint32_t slot = hash32(key) & mask;
+// one value into the table, probing from `slot` on
+__device__ __noinline__ void sp_insert(uint32_t key, long long re, long long im, uint32_t* __restrict__ tkeys,
+                                       unsigned long long* __restrict__ tv, uint32_t slot, uint32_t mask,
+                                       unsigned long long* __restrict__ overflow) {
   for (uint32_t probe = 0; probe <= mask; ++probe) {
     const uint32_t prev = atomicCAS(tkeys + slot, kEmpty, key);
     if (prev == kEmpty || prev == key) {
-      atomicAdd(tv + 2 * slot, (unsigned long long)re);        // two's complement: exact int64 sums
-      atomicAdd(tv + 2 * slot + 1, (unsigned long long)im);
+      sp_add(tv, slot, re, im);
       return;
     }
     slot = (slot + 1) & mask;
@@ -123,64 +130,164 @@ __device__ __forceinline__ void sp_insert(uint32_t key, long long re, long long 
   atomicExch(overflow, 1ull);                                  // table full (cannot happen when sized 2x)
 }
 
-// one qubit level: every entry emits its two children into the table
-__global__ void k_sp_level(const uint32_t* __restrict__ keys, const longlong2* __restrict__ v,
-                           const unsigned long long* __restrict__ count, unsigned long long cap, int n, int beta,
-                           uint32_t* __restrict__ tkeys, unsigned long long* __restrict__ tv, uint32_t mask,
-                           unsigned long long* __restrict__ overflow) {
-  const unsigned long long E = min(*count, cap);
-  for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < E;
-       i += (unsigned long long)gridDim.x * blockDim.x) {
-    const uint32_t k = keys[i];
-    const longlong2 x = v[i];
-    const uint32_t cb = (k >> beta) & 1u, rb = (k >> (n + beta)) & 1u;
-    const uint32_t base = k & ~((1u << beta) | (1u << (n + beta)));
-    const uint32_t kI = base, kX = base | (1u << beta), kY = base | (1u << (n + beta)),
-                   kZ = base | (1u << beta) | (1u << (n + beta));
-    if (rb == cb) {
-      sp_insert(kI, x.x, x.y, tkeys, tv, mask, overflow);                       // I += v
-      if (rb) sp_insert(kZ, -x.x, -x.y, tkeys, tv, mask, overflow);             // Z -= a11
-      else sp_insert(kZ, x.x, x.y, tkeys, tv, mask, overflow);                  // Z += a00
-    } else {
-      sp_insert(kX, x.x, x.y, tkeys, tv, mask, overflow);                       // X += v
-      if (cb) sp_insert(kY, -x.y, x.x, tkeys, tv, mask, overflow);              // Y += i a01
-      else sp_insert(kY, x.y, -x.x, tkeys, tv, mask, overflow);                 // Y -= i a10
-    }
-  }
-}
-
-// nonzero table entries -> the next level's entry list (any order); every
-// slot is cleared after it is read, so the table starts the next level empty
-__global__ void k_sp_compact(uint32_t* __restrict__ tkeys, unsigned long long* __restrict__ tv, uint32_t slots,
-                             uint32_t* __restrict__ keys, longlong2* __restrict__ v,
-                             unsigned long long* __restrict__ count_out, unsigned long long cap,
-                             unsigned long long* __restrict__ overflow) {
-  for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < slots; s += gridDim.x * blockDim.x) {
-    const uint32_t key = tkeys[s];
-    if (key == kEmpty) continue;
-    const long long re = (long long)tv[2 * s], im = (long long)tv[2 * s + 1];
-    tkeys[s] = kEmpty;
-    tv[2 * s] = 0ull;
-    tv[2 * s + 1] = 0ull;
-    if ((re | im) == 0) continue;                              // zero CMW: pruned
-    const unsigned long long pos = atomicAdd(count_out, 1ull);
-    if (pos < cap) { keys[pos] = key; v[pos] = make_longlong2(re, im); }
-    else atomicExch(overflow, 1ull);
-  }
+// Level beta of one entry: its two children into the table.  Both first probes
+// are in flight at once, and no lane waits for another label's: a probe is a
+// round trip to L2, and a level is little else.
+__device__ __forceinline__ void sp_children(uint32_t k, long long re, long long im, int n, int beta,
+                                            uint32_t* __restrict__ tkeys, unsigned long long* __restrict__ tv,
+                                            uint32_t mask, unsigned long long* __restrict__ overflow) {
+  const uint32_t cb = (k >> beta) & 1u, rb = (k >> (n + beta)) & 1u;
+  const uint32_t kI = k & ~((1u << beta) | (1u << (n + beta)));
+  const uint32_t kX = kI | (1u << beta), kY = kI | (1u << (n + beta)), kZ = kX | kY;
+  // I += v and Z +- v (a00 / a11), or X += v and Y +- i v (a01 / a10)
+  const bool diag = rb == cb;
+  const uint32_t k1 = diag ? kI : kX, k2 = diag ? kZ : kY;
+  const long long re2 = diag ? (rb ? -re : re) : (cb ? -im : im);
+  const long long im2 = diag ? (rb ? -im : im) : (cb ? re : -re);
+  const uint32_t s1 = hash32(k1) & mask, s2 = hash32(k2) & mask;
+  const uint32_t p1 = atomicCAS(tkeys + s1, kEmpty, k1);
+  const uint32_t p2 = atomicCAS(tkeys + s2, kEmpty, k2);
+  if (p1 == kEmpty || p1 == k1) sp_add(tv, s1, re, im);
+  else sp_insert(k1, re, im, tkeys, tv, (s1 + 1) & mask, mask, overflow);
+  if (p2 == kEmpty || p2 == k2) sp_add(tv, s2, re2, im2);
+  else sp_insert(k2, re2, im2, tkeys, tv, (s2 + 1) & mask, mask, overflow);
 }
 
 // Counters (unsigned long long): [0] overflow flag, [1 + beta] entries
 // entering level beta (beta = 0..n-1), [1 + n] the final entries.
 constexpr int kSpCounters = 18;                                // n <= 15
 
-// entries of the first level (the input's nonzeros, at most the capacity)
-__global__ void k_sp_start(unsigned long long* ctr, unsigned long long m, unsigned long long cap) {
-  ctr[1] = m < cap ? m : cap;
-  if (m > cap) ctr[0] = 1ull;
+// Slots of the table that level beta fills: twice its children at most.  They
+// are two per entry, and the entries of level beta (counted only while they are
+// read) at most two per entry of the level before, so later levels of a list
+// that shrinks scan, and spread over, a table that shrinks with it (the chain's
+// thirteen: 1.0 million slots each otherwise).
+__device__ __forceinline__ uint32_t sp_slots(const unsigned long long* __restrict__ ctr, int beta, uint32_t slots) {
+  const unsigned long long need = beta == 0 ? 4 * ctr[1] : 8 * ctr[beta];
+  uint32_t p = slots < 1024u ? slots : 1024u;
+  while (p < need && p < slots) p <<= 1;
+  return p;
 }
 
-// status word: TPD_ERR_WORKSPACE (4) if some level had more entries than the capacity
-__global__ void k_sp_status(const unsigned long long* ctr, unsigned* status) { *status = ctr[0] ? 4u : 0u; }
+// the input's entries (key = r*N + c, value on its X-mask's binary point) through level 0
+__global__ void k_sp_first(const int* __restrict__ rows, const int* __restrict__ cols, const double2* __restrict__ vals,
+                           unsigned long long m, unsigned long long cap, int n, const int* __restrict__ emax,
+                           uint32_t* __restrict__ tkeys, unsigned long long* __restrict__ tv, uint32_t slots,
+                           unsigned long long* __restrict__ ctr) {
+  const unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
+  if (i == 0 && m > cap) ctr[0] = 1ull;
+  if (i >= m || i >= cap) return;
+  const uint32_t mask = sp_slots(ctr, 0, slots) - 1;
+  const int r = rows[i], c = cols[i];
+  const int emax_eff = max(emax[(r ^ c) & ((1 << n) - 1)], 1);
+  sp_children(((uint32_t)r << n) | (uint32_t)c, sp_to_fixed(vals[i].x, n, emax_eff), sp_to_fixed(vals[i].y, n, emax_eff),
+              n, 0, tkeys, tv, mask, ctr);
+}
+
+// the entries of the first level (the input's nonzeros, at most the capacity)
+__global__ void k_sp_start(unsigned long long* ctr, unsigned long long m, unsigned long long cap) {
+  ctr[1] = m < cap ? m : cap;
+}
+
+constexpr int kSpThreads = 256;
+constexpr int kSpSlots = 4;                                    // table slots per thread
+
+// The thread's occupied slots of a table, emptied, their zero sums dropped
+// (zero CMWs: pruned); returns how many it keeps in key / re / im.
+__device__ __forceinline__ int sp_take(uint32_t* __restrict__ tkeys, unsigned long long* __restrict__ tv, uint32_t slots,
+                                       uint32_t (&key)[kSpSlots], long long (&re)[kSpSlots], long long (&im)[kSpSlots]) {
+  const unsigned long long s0 = (unsigned long long)blockIdx.x * (kSpThreads * kSpSlots) + threadIdx.x;
+#pragma unroll
+  for (int k = 0; k < kSpSlots; ++k) {
+    const unsigned long long s = s0 + k * kSpThreads;
+    key[k] = s < slots ? tkeys[s] : kEmpty;
+  }
+  // every value in flight before the first slot is emptied
+#pragma unroll
+  for (int k = 0; k < kSpSlots; ++k) {
+    re[k] = im[k] = 0;
+    if (key[k] != kEmpty) {
+      const longlong2 v = *reinterpret_cast<const longlong2*>(tv + 2 * (s0 + k * kSpThreads));
+      re[k] = v.x;
+      im[k] = v.y;
+    }
+  }
+  int kept = 0;
+#pragma unroll
+  for (int k = 0; k < kSpSlots; ++k) {
+    if (key[k] == kEmpty) continue;
+    const unsigned long long s = s0 + k * kSpThreads;
+    tkeys[s] = kEmpty;
+    *reinterpret_cast<ulonglong2*>(tv + 2 * s) = make_ulonglong2(0ull, 0ull);
+    if ((re[k] | im[k]) == 0) key[k] = kEmpty;
+    else ++kept;
+  }
+  return kept;
+}
+
+// The CTA's entries counted into the level's count: their first position,
+// *at the thread's first among them, *total how many; *ok: they fit the capacity.
+__device__ __forceinline__ unsigned long long sp_count(int kept, unsigned long long* __restrict__ count,
+                                                       unsigned long long cap, unsigned long long* __restrict__ overflow,
+                                                       unsigned* at, unsigned* total_out, bool* ok) {
+  __shared__ unsigned part[kSpThreads / 32];
+  __shared__ unsigned long long first;
+  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned inc = (unsigned)kept;
+  for (int d = 1; d < 32; d <<= 1) {
+    const unsigned v = __shfl_up_sync(0xffffffffu, inc, d);
+    if (lane >= (unsigned)d) inc += v;
+  }
+  if (lane == 31) part[warp] = inc;
+  __syncthreads();
+  unsigned before = 0, total = 0;
+  for (unsigned w = 0; w < kSpThreads / 32; ++w) {
+    if (w < warp) before += part[w];
+    total += part[w];
+  }
+  if (threadIdx.x == 0) {
+    first = total ? atomicAdd(count, (unsigned long long)total) : 0ull;
+    if (first + total > cap) atomicExch(overflow, 1ull);
+  }
+  __syncthreads();
+  *ok = first + total <= cap;
+  *at = before + inc - (unsigned)kept;
+  *total_out = total;
+  return first;
+}
+
+// level beta (1..n-1): the entries that level beta - 1 left in one table into
+// the other (count: ctr + 1 + beta)
+__global__ void __launch_bounds__(kSpThreads, 8) k_sp_step(uint32_t* __restrict__ tkeys, unsigned long long* __restrict__ tv,
+                                                        uint32_t slots, unsigned long long* __restrict__ ctr,
+                                                        unsigned long long cap, int n, int beta,
+                                                        uint32_t* __restrict__ ukeys, unsigned long long* __restrict__ uv) {
+  const uint32_t from = sp_slots(ctr, beta - 1, slots);
+  if ((unsigned long long)blockIdx.x * (kSpThreads * kSpSlots) >= from) return;
+  uint32_t key[kSpSlots];
+  long long re[kSpSlots], im[kSpSlots];
+  const int kept = sp_take(tkeys, tv, from, key, re, im);
+  if (!__syncthreads_or(kept)) return;
+  bool ok;
+  unsigned at, total;
+  sp_count(kept, ctr + 1 + beta, cap, ctr, &at, &total, &ok);
+  if (!ok) return;                                             // more entries than the capacity: incomplete
+  // The kept entries side by side, then one a thread: in the table they are
+  // few and far between, and a warp would wait for each of its lanes' slots.
+  __shared__ uint32_t lkey[kSpThreads * kSpSlots];
+  __shared__ longlong2 lval[kSpThreads * kSpSlots];
+#pragma unroll
+  for (int k = 0; k < kSpSlots; ++k)
+    if (key[k] != kEmpty) {
+      lkey[at] = key[k];
+      lval[at] = make_longlong2(re[k], im[k]);
+      ++at;
+    }
+  __syncthreads();
+  const uint32_t mask = sp_slots(ctr, beta, slots) - 1;
+  for (unsigned i = threadIdx.x; i < total; i += kSpThreads)
+    sp_children(lkey[i], lval[i].x, lval[i].y, n, beta, ukeys, uv, mask, ctr);
+}
 
 // RC key -> base-4 string index (bit 2b = c_b, bit 2b+1 = r_b)
 __device__ __forceinline__ unsigned long long sp_string(uint32_t key, int n) {
@@ -192,77 +299,104 @@ __device__ __forceinline__ unsigned long long sp_string(uint32_t key, int n) {
   return s;
 }
 
-// The final entries, sorted by string index: a bitonic sort over the
-// entries padded to Pd = the power of two >= E (padding keys = max), E read on
-// the device.  Steps whose stride is below kSpChunk run inside a CTA on its
-// chunk of the keys in shared memory; the launches for sizes above Pd return
-// at once, so the host plans the launches for the largest possible E.
+// the last level's table -> the final entries (any order) and their sort keys
+__global__ void __launch_bounds__(kSpThreads, 8) k_sp_final(uint32_t* __restrict__ tkeys,
+                                                         unsigned long long* __restrict__ tv, uint32_t slots,
+                                                         unsigned long long* __restrict__ ctr, unsigned long long cap,
+                                                         int n, uint32_t* __restrict__ keys, longlong2* __restrict__ v,
+                                                         unsigned long long* __restrict__ skey,
+                                                         uint32_t* __restrict__ sidx) {
+  const uint32_t from = sp_slots(ctr, n - 1, slots);
+  if ((unsigned long long)blockIdx.x * (kSpThreads * kSpSlots) >= from) return;
+  uint32_t key[kSpSlots];
+  long long re[kSpSlots], im[kSpSlots];
+  const int kept = sp_take(tkeys, tv, from, key, re, im);
+  if (!__syncthreads_or(kept)) return;
+  bool ok;
+  unsigned at, total;
+  unsigned long long pos = sp_count(kept, ctr + 1 + n, cap, ctr, &at, &total, &ok);
+  if (!ok) return;
+  pos += at;
+#pragma unroll
+  for (int k = 0; k < kSpSlots; ++k)
+    if (key[k] != kEmpty) {
+      keys[pos] = key[k];
+      v[pos] = make_longlong2(re[k], im[k]);
+      skey[pos] = sp_string(key[k], n);
+      sidx[pos] = (uint32_t)pos;
+      ++pos;
+    }
+}
+
+
+// The final entries, sorted by string index: a bitonic sort of chunks of
+// kSpChunk keys in shared memory, then merges of pairs of sorted runs, each
+// key to its rank in both, between two buffers.  The number of entries, E, is
+// read on the device: launches for longer runs than there are return at once,
+// so the host plans the launches for the largest possible E.
 constexpr int kSpChunk = 2048;                 // keys per CTA in shared memory
 constexpr int kSpLocalThreads = kSpChunk / 2;  // one compare-exchange pair per thread
 
-__device__ __forceinline__ unsigned long long sp_padded(const unsigned long long* final_count,
-                                                        unsigned long long cap) {
-  const unsigned long long E = min(*final_count, cap);
-  unsigned long long P = 1;
-  while (P < E) P <<= 1;
-  return P;
+// Entries of the final list.  Where a level had more than the capacity (ctr[0])
+// the CTA that passed it wrote none of its own, so the buffers have gaps:
+// there is no list.
+__device__ __forceinline__ unsigned long long sp_entries(const unsigned long long* __restrict__ ctr, int n,
+                                                         unsigned long long cap) {
+  return ctr[0] ? 0ull : min(ctr[1 + n], cap);
 }
 
-// string keys of the final entries into the sort buffer (padding = max)
-__global__ void k_sp_keys(const uint32_t* __restrict__ keys, const unsigned long long* __restrict__ final_count,
-                          unsigned long long cap, int n, unsigned long long* __restrict__ skey,
-                          uint32_t* __restrict__ sidx) {
-  const unsigned long long E = min(*final_count, cap), P = sp_padded(final_count, cap);
-  for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < P;
+// one merge: runs of h keys (the last one shorter) in (skey, sidx) to runs of 2 h in (okey, oidx)
+__global__ void k_sp_merge(const unsigned long long* __restrict__ skey, const uint32_t* __restrict__ sidx,
+                           unsigned long long* __restrict__ okey, uint32_t* __restrict__ oidx,
+                           const unsigned long long* __restrict__ ctr, int n, unsigned long long cap,
+                           unsigned long long h) {
+  const unsigned long long E = sp_entries(ctr, n, cap);
+  if (h >= E) return;
+  for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < E;
        i += (unsigned long long)gridDim.x * blockDim.x) {
-    skey[i] = i < E ? sp_string(keys[i], n) : ~0ull;
-    sidx[i] = (uint32_t)i;
-  }
-}
-
-// one compare-exchange step (j >= kSpChunk, k) over the global buffer
-__global__ void k_sp_bitonic(unsigned long long* __restrict__ skey, uint32_t* __restrict__ sidx,
-                             const unsigned long long* __restrict__ final_count, unsigned long long cap,
-                             unsigned long long j, unsigned long long k) {
-  const unsigned long long P = sp_padded(final_count, cap);
-  if (k > P) return;
-  for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < P;
-       i += (unsigned long long)gridDim.x * blockDim.x) {
-    const unsigned long long l = i ^ j;
-    if (l <= i) continue;
-    const bool up = (i & k) == 0;
-    const unsigned long long a = skey[i], b = skey[l];
-    if ((a > b) == up) {
-      skey[i] = b; skey[l] = a;
-      const uint32_t t = sidx[i]; sidx[i] = sidx[l]; sidx[l] = t;
+    const unsigned long long key = skey[i];
+    const unsigned long long base = i & ~(2 * h - 1), mid = base + h;
+    // keys before this one in the other run (equal keys, from rows or columns
+    // out of range alone: the left run's first), so that every place is taken once
+    const bool left = i < mid;
+    unsigned long long lo = left ? min(mid, E) : base, hi = left ? min(mid + h, E) : mid;
+    const unsigned long long lo0 = lo;
+    while (lo < hi) {
+      const unsigned long long m = (lo + hi) >> 1;
+      if (left ? skey[m] < key : skey[m] <= key) lo = m + 1;
+      else hi = m;
     }
+    const unsigned long long pos = base + (i - (left ? base : mid)) + (lo - lo0);
+    okey[pos] = key;
+    oidx[pos] = sidx[i];
   }
 }
 
-// the steps j < kSpChunk of sizes k in [k_lo, k_hi] on each CTA's chunk, in
-// shared memory (k_lo = 2, k_hi = kSpChunk: the chunks' own sort; k_lo =
-// k_hi = k > kSpChunk: the end of a merge of size k)
+// each CTA's chunk sorted in shared memory (padded with the largest key to a power of two)
 __global__ void __launch_bounds__(kSpLocalThreads) k_sp_local(unsigned long long* __restrict__ skey,
                                                               uint32_t* __restrict__ sidx,
-                                                              const unsigned long long* __restrict__ final_count,
-                                                              unsigned long long cap, unsigned long long k_lo,
-                                                              unsigned long long k_hi) {
+                                                              const unsigned long long* __restrict__ ctr, int n,
+                                                              unsigned long long cap) {
   __shared__ unsigned long long sk[kSpChunk];
   __shared__ uint32_t si[kSpChunk];
-  const unsigned long long P = sp_padded(final_count, cap);
+  const unsigned long long E = sp_entries(ctr, n, cap);
   const unsigned long long base = (unsigned long long)blockIdx.x * kSpChunk;
-  if (base >= P || k_lo > P) return;
-  const unsigned cnt = (unsigned)min((unsigned long long)kSpChunk, P - base);   // a power of two
-  for (unsigned t = threadIdx.x; t < cnt; t += blockDim.x) { sk[t] = skey[base + t]; si[t] = sidx[base + t]; }
+  if (base >= E) return;
+  const unsigned cnt = (unsigned)min((unsigned long long)kSpChunk, E - base);
+  unsigned P = 1;
+  while (P < cnt) P <<= 1;
+  for (unsigned t = threadIdx.x; t < P; t += blockDim.x) {
+    sk[t] = t < cnt ? skey[base + t] : ~0ull;
+    si[t] = t < cnt ? sidx[base + t] : 0u;
+  }
   __syncthreads();
-  const unsigned long long kmax = min(k_hi, P);
-  for (unsigned long long k = k_lo; k <= kmax; k <<= 1) {
-    for (unsigned long long j = min(k >> 1, (unsigned long long)kSpChunk >> 1); j > 0; j >>= 1) {
+  for (unsigned k = 2; k <= P; k <<= 1) {
+    for (unsigned j = k >> 1; j > 0; j >>= 1) {
       const unsigned t = threadIdx.x;
-      const unsigned i = (unsigned)((t / j) * 2 * j + (t % j));
-      const unsigned l = i + (unsigned)j;
-      if (l < cnt) {
-        const bool up = ((base + i) & k) == 0;
+      const unsigned i = (t / j) * 2 * j + (t % j);
+      const unsigned l = i + j;
+      if (l < P) {
+        const bool up = (i & k) == 0;
         const unsigned long long a = sk[i], b = sk[l];
         if ((a > b) == up) {
           sk[i] = b; sk[l] = a;
@@ -275,24 +409,35 @@ __global__ void __launch_bounds__(kSpLocalThreads) k_sp_local(unsigned long long
   for (unsigned t = threadIdx.x; t < cnt; t += blockDim.x) { skey[base + t] = sk[t]; sidx[base + t] = si[t]; }
 }
 
+// the sorted list (after an odd number of merges it is in the second buffer), its length and the status
 __global__ void k_sp_emit(const uint32_t* __restrict__ keys, const longlong2* __restrict__ v,
-                          const unsigned long long* __restrict__ final_count,
-                          unsigned long long cap, const unsigned long long* __restrict__ skey,
-                          const uint32_t* __restrict__ sidx, int n, const int* __restrict__ emax,
-                          unsigned long long capacity, unsigned long long* __restrict__ strings,
-                          double2* __restrict__ weights, unsigned long long* __restrict__ out_count) {
-  const unsigned long long E = min(*final_count, cap);
+                          const unsigned long long* __restrict__ ctr, unsigned long long cap,
+                          const unsigned long long* __restrict__ skey, const uint32_t* __restrict__ sidx,
+                          const unsigned long long* __restrict__ skey2, const uint32_t* __restrict__ sidx2, int n,
+                          const int* __restrict__ emax, unsigned long long capacity,
+                          unsigned long long* __restrict__ strings, double2* __restrict__ weights,
+                          unsigned long long* __restrict__ out_count, unsigned* __restrict__ status) {
+  const unsigned long long E = sp_entries(ctr, n, cap);
+  int merges = 0;
+  for (unsigned long long h = kSpChunk; h < E; h <<= 1) ++merges;
+  if (merges & 1) { skey = skey2; sidx = sidx2; }
   const uint32_t xmask = (1u << n) - 1;
   for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < E && i < capacity;
        i += (unsigned long long)gridDim.x * blockDim.x) {
-    const uint32_t key = keys[sidx[i]];
-    const longlong2 x = v[sidx[i]];
+    const uint32_t at = sidx[i];
+    if (at >= E) continue;                                     // (never: the sort is a permutation)
+    const uint32_t key = keys[at];
+    const longlong2 x = v[at];
     // S_x of the input, and the 1/2 of Eq. 4 per level (the labels keep x = r xor c)
     const int T = 1084 - max(emax[((key >> n) ^ key) & xmask], 1);
     strings[i] = skey[i];
     weights[i] = make_double2(sp_to_double(x.x, T), sp_to_double(x.y, T));
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) *out_count = E;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    *out_count = E;
+    // TPD_ERR_WORKSPACE if some level had more entries than the capacity
+    if (status) *status = ctr[0] ? 4u : 0u;
+  }
 }
 
 unsigned grid_for(unsigned long long items) {
@@ -303,11 +448,13 @@ unsigned grid_for(unsigned long long items) {
 
 }  // namespace
 
-// Workspace: counters | entries (keys, values) | hash table (2x entries,
-// power of two) | sort buffer (power of two >= entries).
+// Workspace: counters, X-mask maxima | two hash tables' keys | their values
+// (2x entries each, power of two) | the final entries and two sort buffers.
+// The first table's values are free once the last level is read (for an even
+// n; the second's for an odd one), and hold the second sort buffer.
 struct SparseLayout {
   size_t ctr, emax, keys, vals, tkeys, tvals, skey, sidx, total;
-  unsigned long long entries, slots, sortn;
+  unsigned long long entries, slots;
 };
 
 static SparseLayout sparse_layout(unsigned long long max_entries) {
@@ -316,17 +463,15 @@ static SparseLayout sparse_layout(unsigned long long max_entries) {
   L.entries = max_entries < 1 ? 1 : max_entries;
   L.slots = 1;
   while (L.slots < 2 * L.entries) L.slots <<= 1;
-  L.sortn = 1;
-  while (L.sortn < L.entries) L.sortn <<= 1;
   size_t off = 0;
   L.ctr = off; off += al(kSpCounters * sizeof(unsigned long long));
   L.emax = off; off += al(sizeof(int) << 15);     // one per X-mask, n <= 15
+  L.tkeys = off; off += al(2 * L.slots * 4);
+  L.tvals = off; off += al(2 * L.slots * 16);
   L.keys = off; off += al(L.entries * 4);
   L.vals = off; off += al(L.entries * 16);
-  L.tkeys = off; off += al(L.slots * 4);
-  L.tvals = off; off += al(L.slots * 16);
-  L.skey = off; off += al(L.sortn * 8);
-  L.sidx = off; off += al(L.sortn * 4);
+  L.skey = off; off += al(L.entries * 8);
+  L.sidx = off; off += al(L.entries * 4);
   L.total = off;
   return L;
 }
@@ -343,42 +488,47 @@ cudaError_t launch_sparse(const int* rows, const int* cols, const void* vals, un
   int* emax = reinterpret_cast<int*>(w + L.emax);
   uint32_t* keys = reinterpret_cast<uint32_t*>(w + L.keys);
   longlong2* v = reinterpret_cast<longlong2*>(w + L.vals);
-  uint32_t* tkeys = reinterpret_cast<uint32_t*>(w + L.tkeys);
-  unsigned long long* tv = reinterpret_cast<unsigned long long*>(w + L.tvals);
+  const uint32_t slots = (uint32_t)L.slots;
+  uint32_t* tkeys[2] = {reinterpret_cast<uint32_t*>(w + L.tkeys), nullptr};
+  unsigned long long* tv[2] = {reinterpret_cast<unsigned long long*>(w + L.tvals), nullptr};
+  tkeys[1] = tkeys[0] + L.slots;
+  tv[1] = tv[0] + 2 * L.slots;
   unsigned long long* skey = reinterpret_cast<unsigned long long*>(w + L.skey);
   uint32_t* sidx = reinterpret_cast<uint32_t*>(w + L.sidx);
   const unsigned long long cap = L.entries;
   cudaError_t e;
-  if ((e = cudaMemsetAsync(w, 0, L.keys, s)) != cudaSuccess) return e;        // counters, X-mask maxima
-  if ((e = cudaMemsetAsync(tkeys, 0xFF, L.slots * 4, s)) != cudaSuccess) return e;   // the table starts empty;
-  if ((e = cudaMemsetAsync(tv, 0, L.slots * 16, s)) != cudaSuccess) return e;        // each level leaves it so
+  // counters and X-mask maxima; both tables start empty, and every read leaves its table so
+  if ((e = cudaMemsetAsync(w, 0, L.tkeys, s)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(tkeys[0], 0xFF, 2 * L.slots * 4, s)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(tv[0], 0, 2 * L.slots * 16, s)) != cudaSuccess) return e;
   const unsigned long long m0 = m < cap ? m : cap;
-  k_sp_start<<<1, 1, 0, s>>>(ctr, m, cap);
   if (m0 > 0) {
-    k_sp_emax<<<grid_for(m0), 256, 0, s>>>(rows, cols, static_cast<const double2*>(vals), m0, n, emax);
-    k_sp_init<<<(unsigned)((m0 + 255) / 256), 256, 0, s>>>(rows, cols, static_cast<const double2*>(vals), m0, n, emax,
-                                                         keys, v);
+    const double2* val = static_cast<const double2*>(vals);
+    k_sp_start<<<1, 1, 0, s>>>(ctr, m, cap);
+    k_sp_emax<<<grid_for(m0), 256, 0, s>>>(rows, cols, val, m0, n, emax);
+    k_sp_first<<<(unsigned)((m0 + 255) / 256), 256, 0, s>>>(rows, cols, val, m, cap, n, emax, tkeys[0], tv[0],
+                                                          slots, ctr);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  const uint32_t mask = (uint32_t)(L.slots - 1);
-  for (int beta = 0; beta < n; ++beta) {
-    k_sp_level<<<grid_for(cap), 256, 0, s>>>(keys, v, ctr + 1 + beta, cap, n, beta, tkeys, tv, mask, ctr);
-    k_sp_compact<<<grid_for(L.slots), 256, 0, s>>>(tkeys, tv, (uint32_t)L.slots, keys, v, ctr + 2 + beta, cap, ctr);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  const unsigned tgrid = (unsigned)((L.slots + kSpThreads * kSpSlots - 1) / (kSpThreads * kSpSlots));
+  for (int beta = 1; beta < n; ++beta) {
+    const int from = (beta - 1) & 1;
+    k_sp_step<<<tgrid, kSpThreads, 0, s>>>(tkeys[from], tv[from], slots, ctr, cap, n, beta, tkeys[from ^ 1],
+                                           tv[from ^ 1]);
   }
-  const unsigned long long* fin = ctr + 1 + n;
-  k_sp_keys<<<grid_for(L.sortn), 256, 0, s>>>(keys, fin, cap, n, skey, sidx);
-  const unsigned chunks = (unsigned)((L.sortn + kSpChunk - 1) / kSpChunk);
-  k_sp_local<<<chunks, kSpLocalThreads, 0, s>>>(skey, sidx, fin, cap, 2, kSpChunk);
-  for (unsigned long long k = 2ull * kSpChunk; k <= L.sortn; k <<= 1) {
-    for (unsigned long long j = k >> 1; j >= (unsigned long long)kSpChunk; j >>= 1)
-      k_sp_bitonic<<<grid_for(L.sortn), 256, 0, s>>>(skey, sidx, fin, cap, j, k);
-    k_sp_local<<<chunks, kSpLocalThreads, 0, s>>>(skey, sidx, fin, cap, k, k);
-  }
-  k_sp_emit<<<grid_for(cap), 256, 0, s>>>(keys, v, fin, cap, skey, sidx, n, emax, capacity, strings,
-                                          static_cast<double2*>(weights), count);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (status) k_sp_status<<<1, 1, 0, s>>>(ctr, status);
+  const int lastt = (n - 1) & 1;                   // the last level's table; the other one is free
+  unsigned long long* skey2 = tv[lastt ^ 1];
+  uint32_t* sidx2 = reinterpret_cast<uint32_t*>(skey2 + L.entries);   // 12 of its 32 bytes per entry
+  k_sp_final<<<tgrid, kSpThreads, 0, s>>>(tkeys[lastt], tv[lastt], slots, ctr, cap, n, keys, v, skey, sidx);
+  const unsigned chunks = (unsigned)((L.entries + kSpChunk - 1) / kSpChunk);
+  k_sp_local<<<chunks, kSpLocalThreads, 0, s>>>(skey, sidx, ctr, n, cap);
+  int at = 0;
+  for (unsigned long long h = kSpChunk; h < L.entries; h <<= 1, at ^= 1)
+    k_sp_merge<<<grid_for(L.entries), 256, 0, s>>>(at ? skey2 : skey, at ? sidx2 : sidx, at ? skey : skey2,
+                                                   at ? sidx : sidx2, ctr, n, cap, h);
+  k_sp_emit<<<grid_for(cap), 256, 0, s>>>(keys, v, ctr, cap, skey, sidx, skey2, sidx2, n, emax, capacity, strings,
+                                          static_cast<double2*>(weights), count, status);
   return cudaGetLastError();
 }
 
