@@ -376,11 +376,17 @@ def _digit_add(x, y, d, n):
     return out
 
 
+def _qudit_passes(n, d):
+    """Passes over the matrix in which the library runs n fused qudit levels."""
+    return -(-n // {2: 4, 3: 3, 4: 2, 5: 2}[d])
+
+
 def time_weyl(tpd, L, torch, stream, d=3, n=9, seed=1006, shifts=8):
     """Decomposition in the Weyl (clock-and-shift) basis of n qudits of
     dimension d (the basis Sec. V names): a random d^n x d^n Hermitian matrix,
-    complex128 (block fixed point, and fp64) and complex64 (fp32), one launch per qudit
-    level, each reading and writing the whole matrix.  Returns the timings
+    complex128 (block fixed point, and fp64) and complex64 (fp32); the fixed
+    point and complex64 run several levels per pass over the matrix, fp64 one
+    launch per level.  Returns the timings
     and, for the accuracy leg, the weights of a few shifts a (row digits b,
     column digits a + b) of each result."""
     from paper_2310_13421_gb300 import synth
@@ -405,9 +411,10 @@ def time_weyl(tpd, L, torch, stream, d=3, n=9, seed=1006, shifts=8):
             assert st == 0, L.status_string(st)
 
         ms = _event_ms(torch, stream, step, setup=lambda: work.copy_(src))
-        alg = 2 * n * N * N * elem
+        passes = n if prec == L.TPD_PREC_PLAIN else _qudit_passes(n, d)
+        alg = 2 * passes * N * N * elem
         out[name] = {"ms": ms, "coeffs_per_s": N * N / (ms * 1e-3), "hbm_gbs_algorithmic": alg / (ms * 1e-3) / 1e9,
-                     "launches": n, "arithmetic": arith}
+                     "launches": passes, "arithmetic": arith}
         rows[name] = work.reshape(-1).index_select(0, torch.from_numpy(pos).cuda()).cpu().numpy() \
             .astype(np.complex128).reshape(len(a_s), N)
         del src, work
@@ -427,8 +434,8 @@ def weyl_accuracy(A, d, a_s, results):
 def time_gellmann(tpd, L, torch, stream, d=3, n=9, seed=1007, labels=256, A=None):
     """Decomposition in the generalized Gell-Mann basis of n qudits of
     dimension d (the other basis Sec. V names): a random d^n x d^n Hermitian
-    matrix (or the given one), complex128 (fp64) and complex64 (fp32), one
-    launch per qudit level, each reading and writing the whole matrix.
+    matrix (or the given one), complex128 (fp64, one launch per qudit level)
+    and complex64 (fp32, several levels per pass over the matrix).
     Returns the timings and, for the accuracy leg, the coefficients of a
     sample of labels (r, c) of each result."""
     from paper_2310_13421_gb300 import synth
@@ -451,10 +458,11 @@ def time_gellmann(tpd, L, torch, stream, d=3, n=9, seed=1007, labels=256, A=None
             assert st == 0, L.status_string(st)
 
         ms = _event_ms(torch, stream, step, setup=lambda: work.copy_(src))
-        alg = 2 * n * N * N * elem
+        passes = n if code == L.TPD_C128 else _qudit_passes(n, d)
+        alg = 2 * passes * N * N * elem
         imag_max = float(work.imag.abs().max().item())
         out[name] = {"ms": ms, "coeffs_per_s": N * N / (ms * 1e-3), "hbm_gbs_algorithmic": alg / (ms * 1e-3) / 1e9,
-                     "launches": n, "arithmetic": arith, "hermitian_input_max_abs_imag": imag_max}
+                     "launches": passes, "arithmetic": arith, "hermitian_input_max_abs_imag": imag_max}
         got[name] = work.reshape(-1).index_select(0, pos.cuda()).cpu().numpy().astype(np.complex128)
         del src, work
         torch.cuda.empty_cache()

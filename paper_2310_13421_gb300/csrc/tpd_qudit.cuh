@@ -1,6 +1,6 @@
-// Several qudit levels of a complex64 decomposition (or composition) in one
-// pass over the matrix: the Weyl (tpd_weyl_c64.cu) and generalized Gell-Mann
-// (tpd_gellmann_c64.cu) bases.
+// Several qudit levels of a complex64 Weyl-basis decomposition (or composition)
+// in one pass over the matrix (tpd_weyl_c64.cu), and the split of n levels into
+// passes that the other qudit kernels share.
 //
 // A level acts on every d x d block of one qudit's row and column digits,
 // all other digits fixed, and the levels of different qudits commute.  A pass
@@ -12,11 +12,10 @@
 // applies the operations, and the roundings, that it applies alone.
 //
 // Why: a level on its own reads and writes the whole matrix, and complex64
-// levels are bound by that traffic (d = 3, n = 9: 1.06 ms a level, 5.86 TB/s),
-// so the passes, not the levels, set the time: d = 3, n = 9 Gell-Mann
-// decomposition 9.53 ms in nine levels and a copy of 0.98 ms before them,
-// 5.13 ms in three passes of three levels, the first reading the input where
-// it is.
+// levels are bound by that traffic, so the passes, not the levels, set the
+// time: d = 3, n = 9 decomposition 9.63 ms in nine levels, 5.07 ms in three
+// passes of three (3.7 TB/s; a capture of the same tiles with the Gell-Mann map
+// had shared-memory wavefronts 60-73 % busy and 77 instructions an element).
 //
 // Tile layout.  k0 > 0 (s >= P): P = d^LP0 consecutive columns share the other
 // digits; an element is at ((i B + j) P + p), B = d^K.  The runs of P
