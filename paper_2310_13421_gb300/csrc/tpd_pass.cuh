@@ -970,8 +970,17 @@ __device__ __forceinline__ void fixed_tile(const G& pd, const PassArgs& args, vo
     // T of a class, -(q_out + out_pow2), falls as its slot rises; zero
     // classes (all of whose sums are 0) round to 0 at any T
     const int tadj = -(kDec ? pd.K : 0) + args.out_pow2;
-    const bool fast = !resid && (slot_hi < slot_lo || (FixedArith::fast_range(-(q_of_slot(slot_hi) + tadj)) &&
-                                                       FixedArith::fast_range(-(q_of_slot(slot_lo) + tadj))));
+    bool fast = !resid && (slot_hi < slot_lo || (FixedArith::fast_range(-(q_of_slot(slot_hi) + tadj)) &&
+                                                 FixedArith::fast_range(-(q_of_slot(slot_lo) + tadj))));
+    if constexpr (!kIntIn) {
+      // a class of IEEE input in slot 0 holds zeros -- or subnormal numbers,
+      // whose sums are not in that range
+      if (zero_slot) {
+#pragma unroll
+        for (int e = 0; e < kElems; ++e)
+          fast &= cls[cl ^ reg_cls(e, l0, l1, l2, l3)] != 0 || (v[e].re | v[e].im) == 0;
+      }
+    }
     // a Hermitian matrix's weights are real, exactly: where a warp's imaginary
     // sums are all 0 they need no conversion (n = 14 last pass 1.74 -> 1.58 ms)
     bool real = false;
