@@ -66,7 +66,8 @@ def _stream(stream):
     return s.cuda_stream
 
 
-_raw_stream = torch._C._cuda_getCurrentRawStream
+# the current stream's handle without a Stream object (absent from builds of torch without CUDA)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 class _enqueue:
