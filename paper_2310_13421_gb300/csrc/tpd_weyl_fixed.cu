@@ -10,12 +10,13 @@
 // double once (RNE).  d = 2, 4: the DFTs are exact (twiddles +-1, +-i) and the
 // 1/d a power of two.  d = 3: with s = x1 + x2, u = x1 - x2,
 //     y0 = x0 + s,   y1,2 = (x0 - s/2) -+ i (sqrt(3)/2) u   (decomposition),
-// s/2 and (sqrt(3)/2) u to a nearby integer; the class's largest component
-// lands in [2^56, 2^57) for K = 3, so a level loses a unit or two of 2^-57 of
+// s/2 toward zero and (sqrt(3)/2) u to the nearest integer; the class's largest
+// component lands in [2^56, 2^57) for K = 3, so a level loses a unit of 2^-57 of
 // it, less than the rounding to double it replaces; 1/3^n is applied once, on the
-// last pass (the passes before take a power of two instead), as a 64-bit
-// fraction before the rounding.  Classes that meet Inf or NaN run IEEE fp64,
-// level by level.
+// last pass (the passes before take a power of two instead), as a 62-bit
+// fraction before the rounding.  Every step is an odd function that keeps zero, so
+// zero sums stay zero, conjugate inputs stay conjugate and -A gives the negated
+// weights.  Classes that meet Inf or NaN run IEEE fp64, level by level.
 //
 // Why: one level a launch converts every element to int64 and back each time
 // and reads and writes the whole matrix (d = 3, n = 9: 2.46 ms a level); a
@@ -40,19 +41,27 @@
 namespace tpd {
 namespace {
 
-// round(sqrt(3) / 2 * 2^64) - 2^64
-constexpr long long kHalfSqrt3 = -2471395088767036514ll;
+// round(sqrt(3) / 2 * 2^62)
+constexpr unsigned long long kHalfSqrt3 = 3993837246235628775ull;
 
-// u c for a fraction c = 1 + cm / 2^64 in [1/2, 1), |u| < 2^63, within three of
-// it and on average at it.  The 32-bit halves' products, without the lowest
-// one, the two in the middle from their high words alone: two wide
-// multiply-adds and two high products (the full 64-bit high product takes over
-// twice the instructions; with it the last pass at d = 3, n = 9 took 3.68 ms).
-__device__ __forceinline__ long long mul_frac(long long u, long long cm) {
-  const int uh = (int)(u >> 32), ch = (int)(cm >> 32);
-  // (+ 1: the two high products lose half a unit each, of two)
-  const int mid = __mulhi(uh, (int)((uint32_t)cm >> 1)) + __mulhi((int)((uint32_t)u >> 1), ch) + 1;
-  return (long long)uh * ch + u + 2ll * mid;
+// The integer nearest to u c, c = C / 2^62 < 1, |u| < 2^62.7: an odd function
+// that keeps 0 (a tie needs u C = 2^61 mod 2^62, for odd C u = +-2^61 alone).
+// With u = 2^32 uh + ul, C = 2^32 ch + cl, the products by the low word of C
+// that are signed take it as cl - 2^32 where cl >= 2^31 (and ch + 1), so that
+// every factor is one 32-bit multiply; the discarded low half of ul cl cannot
+// move the rounding.
+__device__ __forceinline__ long long mul_frac(long long u, unsigned long long C) {
+  const int uh = (int)(u >> 32);
+  const uint32_t ul = (uint32_t)u, ch = (uint32_t)(C >> 32), cl = (uint32_t)C;
+  long long t = (long long)((unsigned long long)ul * ch + __umulhi(ul, cl));
+  t += (long long)uh * (int)cl + (1ll << 29);
+  const long long h = (long long)uh * (int)(ch + (cl >> 31)) + (t >> 32);
+  return (long long)(((unsigned long long)h << 2) | ((uint32_t)t >> 30));
+}
+
+// s / 2 toward zero
+__device__ __forceinline__ long long half_tz(long long s) {
+  return (s + (long long)((unsigned long long)s >> 63)) >> 1;
 }
 
 // headroom bits of K levels, the components below 2^(62 - G): d = 2, 4, sums
@@ -66,7 +75,7 @@ __device__ __forceinline__ bool weyl_fast_range(int T) { return T <= 1022 && T >
 
 struct WeylScale {
   int pow2;            // outputs times 2^pow2 ...
-  long long frac;      // ... times 1 + frac / 2^64 (0: 1) before the rounding ...
+  unsigned long long frac;   // ... times frac / 2^62 (0: 1) before the rounding ...
   double mul;          // ... and times this after it (1 normally)
   double ieee[4];      // the IEEE path's factor of each level of the pass
   double h;            // sqrt(3) / 2
@@ -136,7 +145,7 @@ __device__ __forceinline__ void dft_int(long long (&r)[D], long long (&i)[D]) {
   } else {
     const long long sr = r[1] + r[2], si = i[1] + i[2];
     const long long hr = mul_frac(r[1] - r[2], kHalfSqrt3), hi = mul_frac(i[1] - i[2], kHalfSqrt3);
-    const long long mr = r[0] - (sr >> 1), mi = i[0] - (si >> 1);
+    const long long mr = r[0] - half_tz(sr), mi = i[0] - half_tz(si);
     r[0] += sr; i[0] += si;
     constexpr int p = kDec ? 1 : 2, m = kDec ? 2 : 1;     // p: m - i h u
     r[p] = mr + hi; i[p] = mi - hr;
@@ -417,13 +426,11 @@ cudaError_t run(const double2* src, double2* mat, int n, int d, double last_scal
       sc.pow2 = -take;
       taken += take;
     } else {
-      // 2^taken / 3^n = 2^pow2 (1 + frac / 2^64), the fraction in [1/2, 1)
+      // 2^taken / 3^n = 2^pow2 frac / 2^62, the fraction in [1/2, 1)
       const unsigned long long t3 = ipow(3u, n);
       int e = 0;
       while ((1ull << e) < t3) ++e;                       // 2^(e-1) < 3^n < 2^e
-      // round(2^(e-1) / 3^n 2^64), at least 2^63: as a signed word, the fraction minus one
-      const unsigned __int128 num = (unsigned __int128)1 << (64 + e - 1);
-      sc.frac = (long long)(unsigned long long)((num + t3 / 2) / t3);
+      sc.frac = (unsigned long long)((((unsigned __int128)1 << (62 + e - 1)) + t3 / 2) / t3);
       sc.pow2 = taken - (e - 1);
     }
     cudaError_t e;
