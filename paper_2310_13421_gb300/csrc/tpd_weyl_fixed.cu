@@ -16,7 +16,8 @@
 // last pass (the passes before take a power of two instead), as a 62-bit
 // fraction before the rounding.  Every step is an odd function that keeps zero, so
 // zero sums stay zero, conjugate inputs stay conjugate and -A gives the negated
-// weights.  Classes that meet Inf or NaN run IEEE fp64, level by level.
+// weights.  Classes that meet Inf or NaN run IEEE fp64, level by level, with the
+// same factor a pass (a later class may take elements from both).
 //
 // Why: one level a launch converts every element to int64 and back each time
 // and reads and writes the whole matrix (d = 3, n = 9: 2.46 ms a level); a
@@ -77,7 +78,7 @@ struct WeylScale {
   int pow2;            // outputs times 2^pow2 ...
   unsigned long long frac;   // ... times frac / 2^62 (0: 1) before the rounding ...
   double mul;          // ... and times this after it (1 normally)
-  double ieee[4];      // the IEEE path's factor of each level of the pass
+  double ieee[4];      // the IEEE path's factor of each level of the pass: together the pass's
   double h;            // sqrt(3) / 2
 };
 
@@ -415,15 +416,20 @@ cudaError_t run(const double2* src, double2* mat, int n, int d, double last_scal
     WeylScale sc;
     sc.pow2 = 0; sc.frac = 0; sc.mul = 1.0;
     sc.h = std::sqrt(3.0) * 0.5;
-    for (int m = 0; m < 4; ++m) sc.ieee[m] = kDec ? 1.0 / d : (last && m == K - 1 ? last_scale : 1.0);
+    double whole = 1.0;               // the factor of the pass, on either path (their classes meet in later passes)
     if (!kDec) {
-      if (last) sc.pow2 = split_pow2(last_scale, &sc.mul);
+      if (last) {
+        whole = last_scale;
+        sc.pow2 = split_pow2(last_scale, &sc.mul);
+      }
     } else if (d != 3) {
       sc.pow2 = d == 2 ? -K : -2 * K;
+      whole = std::ldexp(1.0, sc.pow2);
     } else if (!last) {
       // 3^K / 2^sc in [1/2, 1): the values never grow from pass to pass
       const int take = K == 1 ? 2 : (K == 2 ? 4 : 5);
       sc.pow2 = -take;
+      whole = std::ldexp(1.0, -take);
       taken += take;
     } else {
       // 2^taken / 3^n = 2^pow2 frac / 2^62, the fraction in [1/2, 1)
@@ -432,7 +438,13 @@ cudaError_t run(const double2* src, double2* mat, int n, int d, double last_scal
       while ((1ull << e) < t3) ++e;                       // 2^(e-1) < 3^n < 2^e
       sc.frac = (unsigned long long)((((unsigned __int128)1 << (62 + e - 1)) + t3 / 2) / t3);
       sc.pow2 = taken - (e - 1);
+      whole = std::ldexp(1.0, taken) / (double)t3;
     }
+    // (a decomposition's levels before the last by 1/2 or 1/4, exactly: the values never grow)
+    const double each = kDec ? (d == 2 ? 0.5 : 0.25) : 1.0;
+    for (int m = 0; m < 4; ++m) sc.ieee[m] = each;
+    for (int m = 0; m + 1 < K; ++m) whole /= each;
+    sc.ieee[K - 1] = whole;
     cudaError_t e;
     if (p == 0) {
       const First f = pick_first<kDec>(d, K);
