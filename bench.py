@@ -376,9 +376,10 @@ def _digit_add(x, y, d, n):
     return out
 
 
-def _qudit_passes(n, d):
-    """Passes over the matrix in which the library runs n fused qudit levels."""
-    return -(-n // {2: 4, 3: 3, 4: 2, 5: 2}[d])
+def _qudit_passes(n, d, fixed=False):
+    """Passes over the matrix in which the library runs n fused qudit levels
+    (fixed: Weyl complex128 in the block fixed point)."""
+    return -(-n // {2: 4, 3: 2 if fixed else 3, 4: 2, 5: 2}[d])
 
 
 def time_weyl(tpd, L, torch, stream, d=3, n=9, seed=1006, shifts=8):
@@ -411,7 +412,7 @@ def time_weyl(tpd, L, torch, stream, d=3, n=9, seed=1006, shifts=8):
             assert st == 0, L.status_string(st)
 
         ms = _event_ms(torch, stream, step, setup=lambda: work.copy_(src))
-        passes = n if prec == L.TPD_PREC_PLAIN else _qudit_passes(n, d)
+        passes = n if prec == L.TPD_PREC_PLAIN else _qudit_passes(n, d, code == L.TPD_C128)
         alg = 2 * passes * N * N * elem
         out[name] = {"ms": ms, "coeffs_per_s": N * N / (ms * 1e-3), "hbm_gbs_algorithmic": alg / (ms * 1e-3) / 1e9,
                      "launches": passes, "arithmetic": arith}

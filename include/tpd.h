@@ -357,17 +357,18 @@ tpd_status tpd_decompose_coo(const int* rows, const int* cols, const void* value
  *   dtype   TPD_C128 or TPD_C64.
  *   opt     may be NULL (defaults); only opt->precision is read:
  *           DEFAULT / FIXED: complex128 with d <= 4 in a block fixed point --
- *             the d^K elements that the K levels of a pass combine (one
- *             digit-wise cyclic diagonal of a block) on their own binary point
- *             in int64, the DFTs exact for d = 2, 4 and within a few units of
- *             that grid for d = 3 (2^-56 of the largest element), one rounding
- *             to double per output and pass (d = 2, 4 integer inputs: exact);
- *             classes meeting Inf/NaN in IEEE fp64;
+ *             the d elements each DFT combines (one cyclic diagonal of a
+ *             block) on their own binary point in int64 at every level, the
+ *             DFT exact for d = 2, 4 and with sqrt(3) rounded once on that grid
+ *             for d = 3 (3^-n once more, on the last pass's), one rounding to
+ *             double per output and pass (d = 2, 4 integer inputs: exact);
+ *             zero sums stay exactly zero; the elements of a DFT that meet
+ *             Inf/NaN in IEEE fp64;
  *           PLAIN (and DEFAULT for d = 5): IEEE fp64, rounded every level;
  *           complex64: fp32, rounded every level (FIXED and COMPENSATED are
  *           INVALID_ARG for complex64, FIXED for d = 5).
  * One kernel launch per pass of up to 4, 3, 2, 2 levels for d = 2, 3, 4,
- * 5 (complex128 in IEEE fp64: per level).  No workspace; asynchronous on `stream`.
+ * 5 (block fixed point, d = 3: 2 levels; complex128 in IEEE fp64: per level).  No workspace; asynchronous on `stream`.
  * Errors: INVALID_ARG, MISALIGNED, CUDA. */
 tpd_status tpd_weyl_decompose(void* A, int n, int d, int dtype, const tpd_options* opt, void* stream);
 

@@ -4,27 +4,30 @@
 // The K levels of a pass combine only elements whose row digits exceed their
 // column digits by the same a = (a_1..a_K) mod d: a *class*, d^K elements
 // (c + a, c), whose weights Omega_{a,b} go to (b, a + b).  A thread takes one
-// class: it loads the elements, puts them on one binary point in int64 (set by
-// the largest exponent among their components, with headroom for the sums),
-// applies the K levels of d-point DFTs in registers and rounds each output to
-// double once (RNE).  d = 2, 4: the DFTs are exact (twiddles +-1, +-i) and the
-// 1/d a power of two.  d = 3: with s = x1 + x2, u = x1 - x2,
-//     y0 = x0 + s,   y1,2 = (x0 - s/2) -+ i (sqrt(3)/2) u   (decomposition),
-// s/2 toward zero and (sqrt(3)/2) u to the nearest integer; the class's largest
-// component lands in [2^56, 2^57) for K = 3, so a level loses a unit of 2^-57 of
-// it, less than the rounding to double it replaces; 1/3^n is applied once, on the
-// last pass (the passes before take a power of two instead), as a 62-bit
-// fraction before the rounding.  Every step is an odd function that keeps zero, so
-// zero sums stay zero, conjugate inputs stay conjugate and -A gives the negated
-// weights.  Classes that meet Inf or NaN run IEEE fp64, level by level, with the
-// same factor a pass (a later class may take elements from both).
+// class: it loads the elements, applies the K levels of d-point DFTs in
+// registers in int64 and rounds each output to double once (RNE).  At every
+// level the d elements that a DFT adds are on a binary point of their own, set by
+// the largest among them with headroom for the sums -- from the doubles'
+// exponents at the first level, from the leading bits of the sums at the
+// later ones -- so elements that cancel at one level cost the small ones that
+// meet the remainder at the next no bits.  d = 2, 4: the DFTs are exact (twiddles +-1,
+// +-i) and the 1/d a power of two.  d = 3, doubled: with s = x1 + x2, u = x1 - x2,
+//     2 y0 = 2 (x0 + s),   2 y1,2 = (2 x0 - s) -+ i sqrt(3) u   (decomposition),
+// sqrt(3) u to the nearest integer; the largest component lands in [2^58, 2^59).
+// 1/3^n is applied once, on the last pass (the passes before take a power of
+// two instead), as a 62-bit fraction before the rounding.  Every step is an odd
+// function that keeps zero, so zero sums stay zero, conjugate inputs stay
+// conjugate and -A gives the negated weights.  A thread whose class meets Inf or
+// NaN goes level by level, in doubles: the d elements of a DFT in IEEE fp64 if
+// one of them is not finite, else as above, with the same factor a pass (a later
+// class may take elements from both).
 //
 // Why: one level a launch converts every element to int64 and back each time
-// and reads and writes the whole matrix (d = 3, n = 9: 2.46 ms a level); a
-// pass of three levels converts once.  Measured there: 8.9 ms (passes of 3.08,
-// 2.71 and 3.04 ms, 4.0-4.6 TB/s: 138 integer instructions an element at
-// twelve warps an SM, the shift / logic pipe 57 % busy) against 22.1 ms for nine
-// levels and a copy of 1.8 ms before them.
+// and reads and writes the whole matrix (d = 3, n = 9: 2.46 ms a level, 22.1 ms
+// and a copy of 1.8 ms before them); a pass of two converts once.  Measured there:
+// 14.2 ms, passes of 2.8, 3.1, 2.9, 2.8 and (one level and 3^-n) 2.6 ms, bound by
+// integer issue.  With one binary point for a whole class of 27 it was 10.0 ms in
+// three passes, but elements that cancel then took the small ones' low bits along.
 //
 // The outputs of class a go where class -a was read, so the two exchange
 // places: a CTA holds both, one a warp, with a barrier between its loads and
@@ -42,11 +45,25 @@
 namespace tpd {
 namespace {
 
-// round(sqrt(3) / 2 * 2^62)
-constexpr unsigned long long kHalfSqrt3 = 3993837246235628775ull;
+// round(sqrt(3) * 2^62)
+constexpr unsigned long long kSqrt3 = 7987674492471257551ull;
 
-// The integer nearest to u c, c = C / 2^62 < 1, |u| < 2^62.7: an odd function
-// that keeps 0 (a tie needs u C = 2^61 mod 2^62, for odd C u = +-2^61 alone).
+// |v|, with the sign left in `sign` (bit 31)
+__device__ __forceinline__ unsigned long long magnitude(long long v, int& sign) {
+  sign = (int)(v >> 32);
+  asm("{\n\t.reg .pred neg;\n\tsetp.lt.s32 neg, %1, 0;\n\t@neg neg.s64 %0, %0;\n\t}" : "+l"(v) : "r"(sign));
+  return (unsigned long long)v;
+}
+// m 2^-right toward zero with that sign (PTX clamps the amount at 64)
+__device__ __forceinline__ long long shifted_signed(unsigned long long m, int right, int sign) {
+  asm("{\n\t.reg .pred neg;\n\tsetp.lt.s32 neg, %2, 0;\n\tshr.u64 %0, %0, %1;\n\t@neg neg.s64 %0, %0;\n\t}"
+      : "+l"(m) : "r"(right), "r"(sign));
+  return (long long)m;
+}
+
+// The integer nearest to u c, c = C / 2^62, for |u| <= 2^62 and c < 1 or |u| <=
+// 2^60 and c < 2: an odd function that keeps 0 (ties aside, |u| = 2^61 for an odd
+// C: one unit there, which no rounding to double sees for sqrt(3) or 3^-n).
 // With u = 2^32 uh + ul, C = 2^32 ch + cl, the products by the low word of C
 // that are signed take it as cl - 2^32 where cl >= 2^31 (and ch + 1), so that
 // every factor is one 32-bit multiply; the discarded low half of ul cl cannot
@@ -60,32 +77,60 @@ __device__ __forceinline__ long long mul_frac(long long u, unsigned long long C)
   return (long long)(((unsigned long long)h << 2) | ((uint32_t)t >> 30));
 }
 
-// s / 2 toward zero
-__device__ __forceinline__ long long half_tz(long long s) {
-  return (s + (long long)((unsigned long long)s >> 63)) >> 1;
+// Headroom bits of one level: components below 2^(62 - G) give (d = 3: doubled)
+// sums below 2^62.
+template <int D>
+constexpr int kHeadroom = D == 2 ? 1 : (D == 4 ? 2 : 3);
+
+// The d elements that one DFT adds, element c in units of 2^-t[c], onto one
+// binary point, the largest component's leading bit at bit 61 - G (shifted left
+// to bit 62, then right toward zero); returns that point (zeros only: 0).
+template <int D>
+__device__ __forceinline__ int weyl_align(long long (&r)[D], long long (&i)[D], const int (&t)[D]) {
+  constexpr int kZero = 1 << 20;                         // a zero element's place: beyond every other
+  unsigned long long a[D], b[D];
+  int sa[D], sb[D], q[D], lz[D], Q = kZero;
+#pragma unroll
+  for (int c = 0; c < D; ++c) {
+    a[c] = magnitude(r[c], sa[c]);
+    b[c] = magnitude(i[c], sb[c]);
+    const unsigned long long m = a[c] | b[c];
+    lz[c] = __clzll((long long)m);
+    q[c] = m ? t[c] + lz[c] : kZero;
+  }
+#pragma unroll
+  for (int c = 0; c < D; ++c) Q = min(Q, q[c]);
+  const int T = Q - 2 - kHeadroom<D>;
+#pragma unroll
+  for (int c = 0; c < D; ++c) {
+    asm("shl.b64 %0, %0, %1;" : "+l"(a[c]) : "r"(lz[c] - 1));
+    asm("shl.b64 %0, %0, %1;" : "+l"(b[c]) : "r"(lz[c] - 1));
+  }
+#pragma unroll
+  for (int c = 0; c < D; ++c) {
+    r[c] = shifted_signed(a[c], q[c] - Q + 1 + kHeadroom<D>, sa[c]);
+    i[c] = shifted_signed(b[c], q[c] - Q + 1 + kHeadroom<D>, sb[c]);
+  }
+  return Q == kZero ? 0 : T;
 }
 
-// headroom bits of K levels, the components below 2^(62 - G): d = 2, 4, sums
-// of d^K components below 2^62; d = 3, of 3^K sqrt(2) times a component at
-// most, below 2^62.7.
-__host__ __device__ constexpr int weyl_headroom(int d, int K) {
-  return d == 2 ? K : (d == 4 ? 2 * K : (K == 1 ? 2 : (K == 2 ? 3 : 5)));
-}
-// |v| < 2^63 times 2^-T in the normal range, also after rounding up
-__device__ __forceinline__ bool weyl_fast_range(int T) { return T <= 1022 && T >= -960; }
-
+// The factor of a pass: 2^pow2 times frac / 2^62 (0: 1) before the rounding to
+// double, and mul (1 normally) after it.
 struct WeylScale {
-  int pow2;            // outputs times 2^pow2 ...
-  unsigned long long frac;   // ... times frac / 2^62 (0: 1) before the rounding ...
-  double mul;          // ... and times this after it (1 normally)
-  double ieee[4];      // the IEEE path's factor of each level of the pass: together the pass's
+  int pow2;
+  unsigned long long frac;
+  double mul;
+  // level by level (Inf / NaN): levels before the last take 2^each, the last
+  // the rest of pow2 and frac (rest: as one double)
+  int each;
+  double rest;
   double h;            // sqrt(3) / 2
 };
 
-// Class pairs a CTA of a later pass: 128 threads, three CTAs an SM.  Warps that
-// start together share the instruction cache (a class of 27 is ~4,000
-// straight-line instructions): d = 3, n = 9 passes 2.77 / 3.11, 2.71 / 3.04,
-// 2.78 / 3.38, 3.29 / 3.76 ms with 1, 2, 3, 6 (the barrier spans them all).
+// Class pairs a CTA of a later pass: 128 threads.  Warps that start together
+// share the instruction cache (a class is thousands of straight-line
+// instructions), but the barrier spans them all: d = 3, n = 9, two levels at
+// digit stride 81 3.12, 2.88, 3.31, 3.28 ms with 1, 2, 3, 4.
 constexpr int kPairs = 2;
 
 // classes in pairs (a, -a), two self-paired ones together; 255: none
@@ -93,39 +138,6 @@ struct ClassTab {
   uint8_t a[32];
   int units;
 };
-
-// levels of a pass on one class in IEEE arithmetic (Inf / NaN), out of line
-template <int D, int K, bool kDec>
-__device__ __noinline__ void weyl_class_ieee(double2* x, const WeylScale& sc) {
-  constexpr int B = (int)ipow(D, K);
-  Twiddles<double> tw;
-#pragma unroll
-  for (int k = 0; k < D; ++k) {
-    // exact for d = 2, 4; d = 3 uses h alone
-    tw.re[k] = D == 2 ? (k ? -1.0 : 1.0) : (k == 0 ? 1.0 : (k == 2 ? -1.0 : 0.0));
-    tw.im[k] = D == 2 ? 0.0 : (k == 1 ? 1.0 : (k == 3 ? -1.0 : 0.0));
-  }
-  tw.h = sc.h;
-  for (int m = 0, st = 1; m < K; ++m, st *= D)
-    for (int g = 0; g < B / D; ++g) {
-      const int e = (g / st) * (st * D) + g % st;
-      Cx<double> u[D], v[D];
-#pragma unroll
-      for (int c = 0; c < D; ++c) u[c] = {x[e + c * st].x, x[e + c * st].y};
-      dft_ieee<double, D, kDec>(u, v, tw);
-#pragma unroll
-      for (int b = 0; b < D; ++b) x[e + b * st] = make_double2(v[b].re * sc.ieee[m], v[b].im * sc.ieee[m]);
-    }
-}
-
-// outputs outside the normal range, out of line: int64 sums to the doubles' bits
-template <int B>
-__device__ __noinline__ void weyl_class_rare(longlong2* t, int T) {
-  for (int e = 0; e < B; ++e) {
-    t[e].x = __double_as_longlong(FixedArith::to_double_int(t[e].x, T));
-    t[e].y = __double_as_longlong(FixedArith::to_double_int(t[e].y, T));
-  }
-}
 
 // one d-point DFT in int64
 template <int D, bool kDec>
@@ -145,31 +157,120 @@ __device__ __forceinline__ void dft_int(long long (&r)[D], long long (&i)[D]) {
     r[m] = t1r - t3i; i[m] = t1i + t3r;
   } else {
     const long long sr = r[1] + r[2], si = i[1] + i[2];
-    const long long hr = mul_frac(r[1] - r[2], kHalfSqrt3), hi = mul_frac(i[1] - i[2], kHalfSqrt3);
-    const long long mr = r[0] - half_tz(sr), mi = i[0] - half_tz(si);
-    r[0] += sr; i[0] += si;
+    const long long hr = mul_frac(r[1] - r[2], kSqrt3), hi = mul_frac(i[1] - i[2], kSqrt3);
+    const long long mr = 2 * r[0] - sr, mi = 2 * i[0] - si;
+    r[0] = 2 * (r[0] + sr); i[0] = 2 * (i[0] + si);
     constexpr int p = kDec ? 1 : 2, m = kDec ? 2 : 1;     // p: m - i h u
     r[p] = mr + hi; i[p] = mi - hr;
     r[m] = mr - hi; i[m] = mi + hr;
   }
 }
 
-// digit M and above of the class's K levels
+// levels 1 and above of the class; t[e]: the point of element e's sums, kept
+// at the element with digit 0 of the level
 template <int D, int K, bool kDec, int M, int B>
-__device__ __forceinline__ void class_levels(long long (&re)[B], long long (&im)[B]) {
+__device__ __forceinline__ void class_levels(long long (&re)[B], long long (&im)[B], int (&t)[B]) {
   if constexpr (M < K) {
-    constexpr int st = (int)ipow(D, M);
+    constexpr int st = (int)ipow(D, M), before = st / D;  // strides of this level's digit and the last one's
+    int tn[B];
 #pragma unroll
     for (int g = 0; g < B / D; ++g) {
       const int e = (g / st) * (st * D) + g % st;
       long long r[D], i[D];
+      int tc[D];
 #pragma unroll
-      for (int c = 0; c < D; ++c) { r[c] = re[e + c * st]; i[c] = im[e + c * st]; }
+      for (int c = 0; c < D; ++c) {
+        const int x = e + c * st;
+        r[c] = re[x]; i[c] = im[x];
+        tc[c] = t[x - x / before % D * before];
+      }
+      tn[e] = weyl_align<D>(r, i, tc) + (D == 3 ? 1 : 0);
       dft_int<D, kDec>(r, i);
 #pragma unroll
       for (int c = 0; c < D; ++c) { re[e + c * st] = r[c]; im[e + c * st] = i[c]; }
     }
-    class_levels<D, K, kDec, M + 1, B>(re, im);
+#pragma unroll
+    for (int g = 0; g < B / D; ++g) {
+      const int e = (g / st) * (st * D) + g % st;
+      t[e] = tn[e];
+    }
+    class_levels<D, K, kDec, M + 1, B>(re, im, t);
+  }
+}
+
+__device__ __forceinline__ uint32_t exp_field(const double2& x) {
+  return max((uint32_t)__double2hiint(x.x) & 0x7fffffffu, (uint32_t)__double2hiint(x.y) & 0x7fffffffu) >> 20;
+}
+
+// The elements of a DFT, of largest exponent field E, through the first level:
+// onto their binary point, x 2^S with S = 1084 - G - max(E, 1).  Returns the sums' point.
+template <int D, bool kDec>
+__device__ __forceinline__ int first_level(const double2 (&x)[D], int E, long long (&r)[D], long long (&i)[D]) {
+  const int sb = 9 - kHeadroom<D> - max(E, 1);
+#pragma unroll
+  for (int c = 0; c < D; ++c) {
+    r[c] = FixedArith::to_fixed(x[c].x, sb);
+    i[c] = FixedArith::to_fixed(x[c].y, sb);
+  }
+  dft_int<D, kDec>(r, i);
+  return sb + 1075 + (D == 3 ? 1 : 0);
+}
+
+// The levels of a class one after another in doubles, out of line (Inf / NaN).
+template <int D, int K, bool kDec>
+__device__ __noinline__ void weyl_class_levels(double2* x, const WeylScale& sc) {
+  constexpr int B = (int)ipow(D, K);
+  Twiddles<double> tw;
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    // exact for d = 2, 4; d = 3 uses h alone
+    tw.re[k] = D == 2 ? (k ? -1.0 : 1.0) : (k == 0 ? 1.0 : (k == 2 ? -1.0 : 0.0));
+    tw.im[k] = D == 2 ? 0.0 : (k == 1 ? 1.0 : (k == 3 ? -1.0 : 0.0));
+  }
+  tw.h = sc.h;
+  const double each = sc.each == 0 ? 1.0 : (sc.each == -1 ? 0.5 : 0.25);
+  for (int m = 0, st = 1; m < K; ++m, st *= D) {
+    const bool end = m + 1 == K;
+    for (int g = 0; g < B / D; ++g) {
+      const int e = (g / st) * (st * D) + g % st;
+      double2 in[D];
+      uint32_t E = 0;
+#pragma unroll
+      for (int c = 0; c < D; ++c) {
+        in[c] = x[e + c * st];
+        E = max(E, exp_field(in[c]));
+      }
+      if (E == 2047) {
+        Cx<double> u[D], v[D];
+#pragma unroll
+        for (int c = 0; c < D; ++c) u[c] = {in[c].x, in[c].y};
+        dft_ieee<double, D, kDec>(u, v, tw);
+        const double f = end ? sc.rest : each;
+#pragma unroll
+        for (int b = 0; b < D; ++b) x[e + b * st] = make_double2(v[b].re * f, v[b].im * f);
+      } else {
+        long long r[D], i[D];
+        const int T = first_level<D, kDec>(in, (int)E, r, i) - (end ? sc.pow2 - (K - 1) * sc.each : sc.each);
+#pragma unroll
+        for (int b = 0; b < D; ++b) {
+          if (end && sc.frac != 0) {
+            r[b] = mul_frac(r[b], sc.frac);
+            i[b] = mul_frac(i[b], sc.frac);
+          }
+          x[e + b * st] = make_double2(FixedArith::to_double_int(r[b], T) * (end ? sc.mul : 1.0),
+                                       FixedArith::to_double_int(i[b], T) * (end ? sc.mul : 1.0));
+        }
+      }
+    }
+  }
+}
+
+// outputs outside the normal range, out of line: int64 sums to the doubles' bits
+template <int B>
+__device__ __noinline__ void weyl_class_rare(longlong2* v, const int* T) {
+  for (int e = 0; e < B; ++e) {
+    v[e].x = __double_as_longlong(FixedArith::to_double_int(v[e].x, T[e]));
+    v[e].y = __double_as_longlong(FixedArith::to_double_int(v[e].y, T[e]));
   }
 }
 
@@ -206,30 +307,37 @@ struct ClassOffsets {
 // A class in registers: loaded doubles in x (bits), outputs' bits in x.
 template <int D, int K, bool kDec>
 __device__ __forceinline__ void weyl_class(double2 (&x)[ipow(D, K)], const WeylScale& sc) {
-  constexpr int B = (int)ipow(D, K), G = weyl_headroom(D, K);
-  uint32_t h = 0;
+  constexpr int B = (int)ipow(D, K), last = B / D;       // last: stride of the last level's digit
+  uint32_t E[B / D], most = 0;
 #pragma unroll
-  for (int e = 0; e < B; ++e)
-    h = max(h, max((uint32_t)__double2hiint(x[e].x) & 0x7fffffffu, (uint32_t)__double2hiint(x[e].y) & 0x7fffffffu));
-  const int E = (int)(h >> 20);
-  if (E == 2047) {
+  for (int g = 0; g < B / D; ++g) {
+    E[g] = 0;
+#pragma unroll
+    for (int c = 0; c < D; ++c) E[g] = max(E[g], exp_field(x[g * D + c]));
+    most = max(most, E[g]);
+  }
+  if (most == 2047) {
     double2 t[B];
 #pragma unroll
     for (int e = 0; e < B; ++e) t[e] = x[e];
-    weyl_class_ieee<D, K, kDec>(t, sc);
+    weyl_class_levels<D, K, kDec>(t, sc);
 #pragma unroll
     for (int e = 0; e < B; ++e) x[e] = t[e];
     return;
   }
-  // onto the class's binary point: x * 2^S, S = 1084 - G - max(E, 1)
-  const int sb = 9 - G - max(E, 1);
   long long re[B], im[B];
+  int t[B];
 #pragma unroll
-  for (int e = 0; e < B; ++e) {
-    re[e] = FixedArith::to_fixed(x[e].x, sb);
-    im[e] = FixedArith::to_fixed(x[e].y, sb);
+  for (int g = 0; g < B / D; ++g) {
+    double2 in[D];
+    long long r[D], i[D];
+#pragma unroll
+    for (int c = 0; c < D; ++c) in[c] = x[g * D + c];
+    t[g * D] = first_level<D, kDec>(in, (int)E[g], r, i);
+#pragma unroll
+    for (int c = 0; c < D; ++c) { re[g * D + c] = r[c]; im[g * D + c] = i[c]; }
   }
-  class_levels<D, K, kDec, 0, B>(re, im);
+  class_levels<D, K, kDec, 1, B>(re, im, t);
   if (sc.frac != 0) {
 #pragma unroll
     for (int e = 0; e < B; ++e) {
@@ -237,20 +345,29 @@ __device__ __forceinline__ void weyl_class(double2 (&x)[ipow(D, K)], const WeylS
       im[e] = mul_frac(im[e], sc.frac);
     }
   }
-  const int T = sb + 1075 - sc.pow2;                     // value = sum * 2^-T
-  if (weyl_fast_range(T)) {
+  bool fast = true;                                      // value = sum 2^-t
+#pragma unroll
+  for (int e = 0; e < last; ++e) {
+    t[e] -= sc.pow2;
+    fast &= FixedArith::fast_range(t[e]);
+  }
+  if (fast) {
     // real parts through the fp64 conversion unit, imaginary parts through
     // integer instructions (identical roundings): the pipes share the work
 #pragma unroll
     for (int e = 0; e < B; ++e)
-      x[e] = make_double2(FixedArith::to_double_cvt_fast(re[e], T), FixedArith::to_double_fast(im[e], T));
+      x[e] = make_double2(FixedArith::to_double_cvt_fast(re[e], t[e % last]), FixedArith::to_double_fast(im[e], t[e % last]));
   } else {
-    longlong2 t[B];
+    longlong2 v[B];
+    int T[B];
 #pragma unroll
-    for (int e = 0; e < B; ++e) t[e] = make_longlong2(re[e], im[e]);
-    weyl_class_rare<B>(t, T);
+    for (int e = 0; e < B; ++e) {
+      v[e] = make_longlong2(re[e], im[e]);
+      T[e] = t[e % last];
+    }
+    weyl_class_rare<B>(v, T);
 #pragma unroll
-    for (int e = 0; e < B; ++e) x[e] = make_double2(__longlong_as_double(t[e].x), __longlong_as_double(t[e].y));
+    for (int e = 0; e < B; ++e) x[e] = make_double2(__longlong_as_double(v[e].x), __longlong_as_double(v[e].y));
   }
   if (sc.mul != 1.0) {
 #pragma unroll
@@ -289,7 +406,7 @@ __global__ void __launch_bounds__(64 * kPairs, 6 / kPairs)
 // The first pass (s = 1): one group of d^K rows, G groups of d^K columns
 // (fewer in a row group's last tile), every class of them in the CTA.
 template <int D, int K, int G, bool kDec>
-__global__ void __launch_bounds__((ipow(D, K) * G + 31) / 32 * 32, ipow(D, K) * G > 160 ? 2 : 4)
+__global__ void __launch_bounds__((ipow(D, K) * G + 31) / 32 * 32, ipow(D, K) >= 16 ? 3 : 4)
     k_weyl_first(const double2* src, double2* mat, uint32_t N, uint32_t M, uint32_t col_tiles,
                  const __grid_constant__ WeylScale sc) {
   constexpr uint32_t B = ipow(D, K), W = B * G;
@@ -345,9 +462,14 @@ First first() {
   return {k_weyl_first<D, K, G, kDec>, ipow(D, K), (uint32_t)G};
 }
 
-// Column groups of the first pass's tile: what keeps twelve warps an SM busy
-// (d = 3, K = 3: two CTAs of 189 of 192 threads, 82 KB each; 27 elements of 16
-// bytes a thread leave no room for more).
+// Levels per pass at most: one level more adds an alignment and a DFT to every
+// element, one pass more a conversion each way and the matrix's traffic.  d = 3,
+// n = 9: two levels take 2.7-3.2 ms a pass (nine elements a thread, 95
+// registers, twenty warps an SM), three 4.7-5.3 ms (27 elements, 168 registers
+// and spills, twelve warps).
+constexpr int fixed_max_levels(int d) { return d == 3 ? 2 : qudit_max_levels(d); }
+
+// Column groups of the first pass's tile: up to 128 threads a CTA.
 template <bool kDec>
 First pick_first(int d, int K) {
   switch (d * 8 + K) {
@@ -355,7 +477,6 @@ First pick_first(int d, int K) {
     case 2 * 8 + 3: return first<2, 3, 16, kDec>();
     case 2 * 8 + 2: return first<2, 2, 8, kDec>();
     case 2 * 8 + 1: return first<2, 1, 16, kDec>();
-    case 3 * 8 + 3: return first<3, 3, 7, kDec>();
     case 3 * 8 + 2: return first<3, 2, 14, kDec>();
     case 3 * 8 + 1: return first<3, 1, 10, kDec>();
     case 4 * 8 + 2: return first<4, 2, 8, kDec>();
@@ -369,8 +490,8 @@ PassFn pick_pass(int d, int K) {
     case 2 * 8 + 4: return k_weyl_class<2, 4, kDec>;
     case 2 * 8 + 3: return k_weyl_class<2, 3, kDec>;
     case 2 * 8 + 2: return k_weyl_class<2, 2, kDec>;
-    case 3 * 8 + 3: return k_weyl_class<3, 3, kDec>;
     case 3 * 8 + 2: return k_weyl_class<3, 2, kDec>;
+    case 3 * 8 + 1: return k_weyl_class<3, 1, kDec>;
     case 4 * 8 + 2: return k_weyl_class<4, 2, kDec>;
     default: return k_weyl_class<4, 1, kDec>;
   }
@@ -408,7 +529,7 @@ int split_pow2(double v, double* resid) {
 template <bool kDec>
 cudaError_t run(const double2* src, double2* mat, int n, int d, double last_scale, cudaStream_t st) {
   const uint32_t N = ipow((uint32_t)d, n);
-  const int most = qudit_max_levels(d), passes = (n + most - 1) / most;
+  const int most = fixed_max_levels(d), passes = (n + most - 1) / most;
   int k0 = 0, taken = 0;             // taken: powers of two applied by the passes so far (d = 3)
   for (int p = 0; p < passes; ++p) {
     const int K = n / passes + (p < n % passes ? 1 : 0);
@@ -426,11 +547,11 @@ cudaError_t run(const double2* src, double2* mat, int n, int d, double last_scal
       sc.pow2 = d == 2 ? -K : -2 * K;
       whole = std::ldexp(1.0, sc.pow2);
     } else if (!last) {
-      // 3^K / 2^sc in [1/2, 1): the values never grow from pass to pass
-      const int take = K == 1 ? 2 : (K == 2 ? 4 : 5);
-      sc.pow2 = -take;
-      whole = std::ldexp(1.0, -take);
-      taken += take;
+      // 3^levels / 2^taken in [1/2, 1): the values never grow beyond the input's, nor shrink much below
+      sc.pow2 = taken;
+      while ((1u << taken) < ipow(3u, k0 + K)) ++taken;
+      sc.pow2 -= taken;
+      whole = std::ldexp(1.0, sc.pow2);
     } else {
       // 2^taken / 3^n = 2^pow2 frac / 2^62, the fraction in [1/2, 1)
       const unsigned long long t3 = ipow(3u, n);
@@ -441,10 +562,8 @@ cudaError_t run(const double2* src, double2* mat, int n, int d, double last_scal
       whole = std::ldexp(1.0, taken) / (double)t3;
     }
     // (a decomposition's levels before the last by 1/2 or 1/4, exactly: the values never grow)
-    const double each = kDec ? (d == 2 ? 0.5 : 0.25) : 1.0;
-    for (int m = 0; m < 4; ++m) sc.ieee[m] = each;
-    for (int m = 0; m + 1 < K; ++m) whole /= each;
-    sc.ieee[K - 1] = whole;
+    sc.each = kDec ? (d == 2 ? -1 : -2) : 0;
+    sc.rest = std::ldexp(whole, -(K - 1) * sc.each);
     cudaError_t e;
     if (p == 0) {
       const First f = pick_first<kDec>(d, K);
@@ -455,8 +574,8 @@ cudaError_t run(const double2* src, double2* mat, int n, int d, double last_scal
     } else {
       const uint32_t M = N / ipow((uint32_t)d, K), nq = M * M;
       const ClassTab tab = class_pairs(d, K);
-      pick_pass<kDec>(d, K)<<<dim3((nq + 32 * kPairs - 1) / (32 * kPairs), (unsigned)tab.units), 64 * kPairs, 0, st>>>(mat, N, ipow((uint32_t)d, k0), M,
-                                                                                       nq, tab, sc);
+      const dim3 grid((nq + 32 * kPairs - 1) / (32 * kPairs), (unsigned)tab.units);
+      pick_pass<kDec>(d, K)<<<grid, 64 * kPairs, 0, st>>>(mat, N, ipow((uint32_t)d, k0), M, nq, tab, sc);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k0 += K;
