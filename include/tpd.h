@@ -320,8 +320,9 @@ tpd_status tpd_nonzero_write(const void* W, int n, int dtype, double tol, unsign
  *   n           1..15.
  *   max_entries the most entries any level may hold (device memory grows with
  *               it: 112 to 192 bytes per entry); more sets *status to
- *               TPD_ERR_WORKSPACE and the list is empty (*count = 0).  A level holds
- *               at most 2x the entries of the one before.
+ *               TPD_ERR_WORKSPACE and the list is incomplete: what is left of the
+ *               entries that fitted, sorted, *count <= max_entries of them.
+ *               A level holds at most 2x the entries of the one before.
  *   strings, weights, capacity, count   as tpd_nonzero_list.
  *   status      device, one unsigned (may be NULL): TPD_OK or TPD_ERR_WORKSPACE.
  *   workspace   device, tpd_sparse_workspace_size(max_entries) bytes, 256-byte aligned.

@@ -226,10 +226,12 @@ __device__ __forceinline__ int sp_take(uint32_t* __restrict__ tkeys, unsigned lo
 }
 
 // The CTA's entries counted into the level's count: their first position,
-// *at the thread's first among them, *total how many; *ok: they fit the capacity.
+// *at the thread's first among them, *fit how many the capacity has room for.
+// The CTAs' positions follow one another, so the entries below the capacity
+// have no gaps.
 __device__ __forceinline__ unsigned long long sp_count(int kept, unsigned long long* __restrict__ count,
                                                        unsigned long long cap, unsigned long long* __restrict__ overflow,
-                                                       unsigned* at, unsigned* total_out, bool* ok) {
+                                                       unsigned* at, unsigned* fit) {
   __shared__ unsigned part[kSpThreads / 32];
   __shared__ unsigned long long first;
   const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -250,9 +252,8 @@ __device__ __forceinline__ unsigned long long sp_count(int kept, unsigned long l
     if (first + total > cap) atomicExch(overflow, 1ull);
   }
   __syncthreads();
-  *ok = first + total <= cap;
   *at = before + inc - (unsigned)kept;
-  *total_out = total;
+  *fit = first >= cap ? 0u : (unsigned)min((unsigned long long)total, cap - first);
   return first;
 }
 
@@ -268,10 +269,8 @@ __global__ void __launch_bounds__(kSpThreads, 8) k_sp_step(uint32_t* __restrict_
   long long re[kSpSlots], im[kSpSlots];
   const int kept = sp_take(tkeys, tv, from, key, re, im);
   if (!__syncthreads_or(kept)) return;
-  bool ok;
-  unsigned at, total;
-  sp_count(kept, ctr + 1 + beta, cap, ctr, &at, &total, &ok);
-  if (!ok) return;                                             // more entries than the capacity: incomplete
+  unsigned at, fit;
+  sp_count(kept, ctr + 1 + beta, cap, ctr, &at, &fit);        // entries past the capacity are lost (the status says so)
   // The kept entries side by side, then one a thread: in the table they are
   // few and far between, and a warp would wait for each of its lanes' slots.
   __shared__ uint32_t lkey[kSpThreads * kSpSlots];
@@ -285,7 +284,7 @@ __global__ void __launch_bounds__(kSpThreads, 8) k_sp_step(uint32_t* __restrict_
     }
   __syncthreads();
   const uint32_t mask = sp_slots(ctr, beta, slots) - 1;
-  for (unsigned i = threadIdx.x; i < total; i += kSpThreads)
+  for (unsigned i = threadIdx.x; i < fit; i += kSpThreads)
     sp_children(lkey[i], lval[i].x, lval[i].y, n, beta, ukeys, uv, mask, ctr);
 }
 
@@ -312,14 +311,11 @@ __global__ void __launch_bounds__(kSpThreads, 8) k_sp_final(uint32_t* __restrict
   long long re[kSpSlots], im[kSpSlots];
   const int kept = sp_take(tkeys, tv, from, key, re, im);
   if (!__syncthreads_or(kept)) return;
-  bool ok;
-  unsigned at, total;
-  unsigned long long pos = sp_count(kept, ctr + 1 + n, cap, ctr, &at, &total, &ok);
-  if (!ok) return;
-  pos += at;
+  unsigned at, fit;
+  unsigned long long pos = sp_count(kept, ctr + 1 + n, cap, ctr, &at, &fit) + at;
 #pragma unroll
   for (int k = 0; k < kSpSlots; ++k)
-    if (key[k] != kEmpty) {
+    if (key[k] != kEmpty && pos < cap) {
       keys[pos] = key[k];
       v[pos] = make_longlong2(re[k], im[k]);
       skey[pos] = sp_string(key[k], n);
@@ -337,12 +333,10 @@ __global__ void __launch_bounds__(kSpThreads, 8) k_sp_final(uint32_t* __restrict
 constexpr int kSpChunk = 2048;                 // keys per CTA in shared memory
 constexpr int kSpLocalThreads = kSpChunk / 2;  // one compare-exchange pair per thread
 
-// Entries of the final list.  Where a level had more than the capacity (ctr[0])
-// the CTA that passed it wrote none of its own, so the buffers have gaps:
-// there is no list.
+// entries of the final list: those that fit
 __device__ __forceinline__ unsigned long long sp_entries(const unsigned long long* __restrict__ ctr, int n,
                                                          unsigned long long cap) {
-  return ctr[0] ? 0ull : min(ctr[1 + n], cap);
+  return min(ctr[1 + n], cap);
 }
 
 // one merge: runs of h keys (the last one shorter) in (skey, sidx) to runs of 2 h in (okey, oidx)
