@@ -115,17 +115,21 @@ __device__ __forceinline__ void sp_add(unsigned long long* __restrict__ tv, uint
   atomicAdd(tv + 2ull * slot + 1, (unsigned long long)im);
 }
 
+// a key's first slot of a table of any size, and the slot after another
+__device__ __forceinline__ uint32_t sp_slot(uint32_t key, uint32_t slots) { return __umulhi(hash32(key), slots); }
+__device__ __forceinline__ uint32_t sp_next(uint32_t slot, uint32_t slots) { return slot + 1 == slots ? 0u : slot + 1; }
+
 // one value into the table, probing from `slot` on
 __device__ __noinline__ void sp_insert(uint32_t key, long long re, long long im, uint32_t* __restrict__ tkeys,
-                                       unsigned long long* __restrict__ tv, uint32_t slot, uint32_t mask,
+                                       unsigned long long* __restrict__ tv, uint32_t slot, uint32_t slots,
                                        unsigned long long* __restrict__ overflow) {
-  for (uint32_t probe = 0; probe <= mask; ++probe) {
+  for (uint32_t probe = 0; probe < slots; ++probe) {
     const uint32_t prev = atomicCAS(tkeys + slot, kEmpty, key);
     if (prev == kEmpty || prev == key) {
       sp_add(tv, slot, re, im);
       return;
     }
-    slot = (slot + 1) & mask;
+    slot = sp_next(slot, slots);
   }
   atomicExch(overflow, 1ull);                                  // table full (cannot happen when sized 2x)
 }
@@ -135,7 +139,7 @@ __device__ __noinline__ void sp_insert(uint32_t key, long long re, long long im,
 // round trip to L2, and a level is little else.
 __device__ __forceinline__ void sp_children(uint32_t k, long long re, long long im, int n, int beta,
                                             uint32_t* __restrict__ tkeys, unsigned long long* __restrict__ tv,
-                                            uint32_t mask, unsigned long long* __restrict__ overflow) {
+                                            uint32_t slots, unsigned long long* __restrict__ overflow) {
   const uint32_t cb = (k >> beta) & 1u, rb = (k >> (n + beta)) & 1u;
   const uint32_t kI = k & ~((1u << beta) | (1u << (n + beta)));
   const uint32_t kX = kI | (1u << beta), kY = kI | (1u << (n + beta)), kZ = kX | kY;
@@ -144,13 +148,13 @@ __device__ __forceinline__ void sp_children(uint32_t k, long long re, long long 
   const uint32_t k1 = diag ? kI : kX, k2 = diag ? kZ : kY;
   const long long re2 = diag ? (rb ? -re : re) : (cb ? -im : im);
   const long long im2 = diag ? (rb ? -im : im) : (cb ? re : -re);
-  const uint32_t s1 = hash32(k1) & mask, s2 = hash32(k2) & mask;
+  const uint32_t s1 = sp_slot(k1, slots), s2 = sp_slot(k2, slots);
   const uint32_t p1 = atomicCAS(tkeys + s1, kEmpty, k1);
   const uint32_t p2 = atomicCAS(tkeys + s2, kEmpty, k2);
   if (p1 == kEmpty || p1 == k1) sp_add(tv, s1, re, im);
-  else sp_insert(k1, re, im, tkeys, tv, (s1 + 1) & mask, mask, overflow);
+  else sp_insert(k1, re, im, tkeys, tv, sp_next(s1, slots), slots, overflow);
   if (p2 == kEmpty || p2 == k2) sp_add(tv, s2, re2, im2);
-  else sp_insert(k2, re2, im2, tkeys, tv, (s2 + 1) & mask, mask, overflow);
+  else sp_insert(k2, re2, im2, tkeys, tv, sp_next(s2, slots), slots, overflow);
 }
 
 // Counters (unsigned long long): [0] overflow flag, [1 + beta] entries
@@ -164,9 +168,9 @@ constexpr int kSpCounters = 18;                                // n <= 15
 // thirteen: 1.0 million slots each otherwise).
 __device__ __forceinline__ uint32_t sp_slots(const unsigned long long* __restrict__ ctr, int beta, uint32_t slots) {
   const unsigned long long need = beta == 0 ? 4 * ctr[1] : 8 * ctr[beta];
-  uint32_t p = slots < 1024u ? slots : 1024u;
+  unsigned long long p = 1024;
   while (p < need && p < slots) p <<= 1;
-  return p;
+  return p < slots ? (uint32_t)p : slots;
 }
 
 // the input's entries (key = r*N + c, value on its X-mask's binary point) through level 0
@@ -177,11 +181,11 @@ __global__ void k_sp_first(const int* __restrict__ rows, const int* __restrict__
   const unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
   if (i == 0 && m > cap) ctr[0] = 1ull;
   if (i >= m || i >= cap) return;
-  const uint32_t mask = sp_slots(ctr, 0, slots) - 1;
+  const uint32_t size = sp_slots(ctr, 0, slots);
   const int r = rows[i], c = cols[i];
   const int emax_eff = max(emax[(r ^ c) & ((1 << n) - 1)], 1);
   sp_children(((uint32_t)r << n) | (uint32_t)c, sp_to_fixed(vals[i].x, n, emax_eff), sp_to_fixed(vals[i].y, n, emax_eff),
-              n, 0, tkeys, tv, mask, ctr);
+              n, 0, tkeys, tv, size, ctr);
 }
 
 // the entries of the first level (the input's nonzeros, at most the capacity)
@@ -283,9 +287,9 @@ __global__ void __launch_bounds__(kSpThreads, 8) k_sp_step(uint32_t* __restrict_
       ++at;
     }
   __syncthreads();
-  const uint32_t mask = sp_slots(ctr, beta, slots) - 1;
+  const uint32_t size = sp_slots(ctr, beta, slots);
   for (unsigned i = threadIdx.x; i < fit; i += kSpThreads)
-    sp_children(lkey[i], lval[i].x, lval[i].y, n, beta, ukeys, uv, mask, ctr);
+    sp_children(lkey[i], lval[i].x, lval[i].y, n, beta, ukeys, uv, size, ctr);
 }
 
 // RC key -> base-4 string index (bit 2b = c_b, bit 2b+1 = r_b)
@@ -442,12 +446,13 @@ unsigned grid_for(unsigned long long items) {
 
 }  // namespace
 
-// Workspace: counters, X-mask maxima | two hash tables' keys | their values
-// (2x entries each, power of two) | the final entries and two sort buffers.
-// The first table's values are free once the last level is read (for an even
-// n; the second's for an odd one), and hold the second sort buffer.
+// Workspace: counters, X-mask maxima | two hash tables' keys | their values (two
+// slots an entry each: a level holds at most twice the entries of the one
+// before).  The last level leaves one table to be read and one free: the final
+// entries and their sort keys go into the free one's values (32 bytes an
+// entry, all of them), the second sort buffer into the other's, empty by then.
 struct SparseLayout {
-  size_t ctr, emax, keys, vals, tkeys, tvals, skey, sidx, total;
+  size_t ctr, emax, tkeys, tvals, total;
   unsigned long long entries, slots;
 };
 
@@ -455,17 +460,12 @@ static SparseLayout sparse_layout(unsigned long long max_entries) {
   auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
   SparseLayout L;
   L.entries = max_entries < 1 ? 1 : max_entries;
-  L.slots = 1;
-  while (L.slots < 2 * L.entries) L.slots <<= 1;
+  L.slots = 2 * L.entries;
   size_t off = 0;
   L.ctr = off; off += al(kSpCounters * sizeof(unsigned long long));
   L.emax = off; off += al(sizeof(int) << 15);     // one per X-mask, n <= 15
   L.tkeys = off; off += al(2 * L.slots * 4);
   L.tvals = off; off += al(2 * L.slots * 16);
-  L.keys = off; off += al(L.entries * 4);
-  L.vals = off; off += al(L.entries * 16);
-  L.skey = off; off += al(L.entries * 8);
-  L.sidx = off; off += al(L.entries * 4);
   L.total = off;
   return L;
 }
@@ -480,15 +480,11 @@ cudaError_t launch_sparse(const int* rows, const int* cols, const void* vals, un
   char* w = static_cast<char*>(ws);
   unsigned long long* ctr = reinterpret_cast<unsigned long long*>(w + L.ctr);   // see kSpCounters
   int* emax = reinterpret_cast<int*>(w + L.emax);
-  uint32_t* keys = reinterpret_cast<uint32_t*>(w + L.keys);
-  longlong2* v = reinterpret_cast<longlong2*>(w + L.vals);
   const uint32_t slots = (uint32_t)L.slots;
   uint32_t* tkeys[2] = {reinterpret_cast<uint32_t*>(w + L.tkeys), nullptr};
   unsigned long long* tv[2] = {reinterpret_cast<unsigned long long*>(w + L.tvals), nullptr};
   tkeys[1] = tkeys[0] + L.slots;
   tv[1] = tv[0] + 2 * L.slots;
-  unsigned long long* skey = reinterpret_cast<unsigned long long*>(w + L.skey);
-  uint32_t* sidx = reinterpret_cast<uint32_t*>(w + L.sidx);
   const unsigned long long cap = L.entries;
   cudaError_t e;
   // counters and X-mask maxima; both tables start empty, and every read leaves its table so
@@ -512,8 +508,12 @@ cudaError_t launch_sparse(const int* rows, const int* cols, const void* vals, un
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const int lastt = (n - 1) & 1;                   // the last level's table; the other one is free
-  unsigned long long* skey2 = tv[lastt ^ 1];
-  uint32_t* sidx2 = reinterpret_cast<uint32_t*>(skey2 + L.entries);   // 12 of its 32 bytes per entry
+  longlong2* v = reinterpret_cast<longlong2*>(tv[lastt ^ 1]);
+  unsigned long long* skey = reinterpret_cast<unsigned long long*>(v + L.entries);
+  uint32_t* keys = reinterpret_cast<uint32_t*>(skey + L.entries);
+  uint32_t* sidx = keys + L.entries;
+  unsigned long long* skey2 = tv[lastt];           // once k_sp_final has read it
+  uint32_t* sidx2 = reinterpret_cast<uint32_t*>(skey2 + L.entries);
   k_sp_final<<<tgrid, kSpThreads, 0, s>>>(tkeys[lastt], tv[lastt], slots, ctr, cap, n, keys, v, skey, sidx);
   const unsigned chunks = (unsigned)((L.entries + kSpChunk - 1) / kSpChunk);
   k_sp_local<<<chunks, kSpLocalThreads, 0, s>>>(skey, sidx, ctr, n, cap);
