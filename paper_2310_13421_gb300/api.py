@@ -50,11 +50,13 @@ def _check_device(t):
 def _target(A, inplace):
     """(input, output) of a call on A.  In place: A itself.  Else a new output,
     with A read where it is -- or, where A cannot be (a lazily conjugated or
-    negated view, memory not aligned to its elements, a tensor whose copy
-    autograd follows), a copy of it that is then worked on in place."""
+    negated view, zeros without memory, memory not aligned to its elements, a
+    tensor whose copy autograd follows), a copy of it that is then worked on in
+    place."""
     if inplace:
         return A, A
-    if (A.is_conj() or A.is_neg() or A.data_ptr() % A.element_size() or (A.requires_grad and torch.is_grad_enabled())
+    p = A.data_ptr()
+    if (A.is_conj() or A.is_neg() or p == 0 or p % A.element_size() or (A.requires_grad and torch.is_grad_enabled())
             or torch.autograd.forward_ad._current_level >= 0):
         out = A.clone()
         return out, out

@@ -1,0 +1,36 @@
+"""CPU: which inputs an out-of-place call reads where they are, and which it copies
+first."""
+import pytest
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def api():
+    from paper_2310_13421_gb300 import api as a
+    return a
+
+
+def _copied(api, A):
+    src, out = api._target(A, False)
+    assert out.data_ptr() not in (0, A.data_ptr()) and out.shape == A.shape and out.dtype == A.dtype
+    assert src is A or src is out
+    return src is out
+
+
+def test_plain_inputs_are_read_in_place(api):
+    A = torch.randn(8, 8, dtype=torch.complex128)
+    assert not _copied(api, A) and not _copied(api, A.detach())
+    assert api._target(A, True) == (A, A)
+
+
+def test_lazy_and_followed_inputs_are_copied(api):
+    A = torch.randn(8, 8, dtype=torch.complex128)
+    assert _copied(api, A.conj()) and _copied(api, A.clone().requires_grad_())
+    with torch.no_grad():
+        assert not _copied(api, A.clone().requires_grad_())
+
+
+def test_zeros_without_memory_are_copied(api):
+    Z = torch._efficientzerotensor((8, 8), dtype=torch.complex128)
+    assert Z.data_ptr() == 0 and _copied(api, Z)
