@@ -122,10 +122,17 @@ def make_options(precision=None, skip_zero=False, tile_bits=0, max_levels=0, var
     return L.options(precision, skip_zero, tile_bits, max_levels, variant, l2_chunk_mb=l2_chunk_mb)
 
 
-@functools.lru_cache(maxsize=256)
 def _options(precision, skip_zero=False, tile_bits=0, max_levels=0, variant=0, l2_chunk_mb=0):
-    """make_options for the library's own calls, which only read the struct."""
-    return make_options(precision, skip_zero, tile_bits, max_levels, variant, l2_chunk_mb)
+    """make_options for the library's own calls, which only read the struct:
+    kept by value (the arguments may be anything that converts)."""
+    if isinstance(precision, str) or precision is None:
+        precision = _PREC[precision]
+    return _options_of(int(precision), bool(skip_zero), int(tile_bits), int(max_levels), int(variant), int(l2_chunk_mb))
+
+
+@functools.lru_cache(maxsize=256)
+def _options_of(*values):
+    return make_options(*values)
 
 
 def workspace_size(n, dtype, **kw):

@@ -34,3 +34,18 @@ def test_lazy_and_followed_inputs_are_copied(api):
 def test_zeros_without_memory_are_copied(api):
     Z = torch._efficientzerotensor((8, 8), dtype=torch.complex128)
     assert Z.data_ptr() == 0 and _copied(api, Z)
+
+
+def test_options_by_value(api):
+    # anything that converts to a number, also what cannot be hashed or changes later
+    import numpy as np
+    t = torch.tensor(11)
+    assert api._options("fixed", tile_bits=t).tile_bits == 11
+    t += 1
+    assert api._options("fixed", tile_bits=t).tile_bits == 12
+    o = api._options(np.array(0), np.bool_(True), np.array(12), 3.0, variant=np.int64(1))
+    assert (o.skip_zero, o.tile_bits, o.max_levels, o.variant) == (1, 12, 3, 1)
+    assert api._options(None) is api._options("default")
+    for bad in ("exact", "Fixed"):
+        with pytest.raises(KeyError):
+            api._options(bad)
