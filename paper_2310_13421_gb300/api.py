@@ -57,7 +57,7 @@ def _target(A, inplace):
         return A, A
     p = A.data_ptr()
     if (A.is_conj() or A.is_neg() or p == 0 or p % A.element_size() or (A.requires_grad and torch.is_grad_enabled())
-            or torch.autograd.forward_ad._current_level >= 0):
+            or getattr(torch.autograd.forward_ad, "_current_level", 0) >= 0):   # (a torch without it: copied)
         out = A.clone()
         return out, out
     return A, torch.empty_like(A)
@@ -68,7 +68,7 @@ def _stream(stream):
     return s.cuda_stream
 
 
-# the current stream's handle without a Stream object (absent from builds of torch without CUDA)
+# the current stream's handle without a Stream object; None where torch has no such function
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
@@ -91,7 +91,7 @@ class _enqueue:
         self.device, self.stream, self.inputs, self.entered = device, stream, inputs, None
 
     def __enter__(self):
-        if self.stream is None and self.device.index == torch.cuda.current_device():
+        if self.stream is None and _raw_stream is not None and self.device.index == torch.cuda.current_device():
             return _raw_stream(self.device.index)
         self.entered = contextlib.ExitStack()
         self.entered.enter_context(torch.cuda.device(self.device))

@@ -49,3 +49,31 @@ def test_options_by_value(api):
     for bad in ("exact", "Fixed"):
         with pytest.raises(KeyError):
             api._options(bad)
+
+
+def test_without_the_forward_mode_level_inputs_are_copied(api, monkeypatch):
+    monkeypatch.delattr(torch.autograd.forward_ad, "_current_level")
+    assert _copied(api, torch.randn(8, 8, dtype=torch.complex128))
+
+
+def test_without_the_raw_stream_function_the_stream_is_entered(api, monkeypatch):
+    class Stream:
+        cuda_stream = 77
+
+    class Entered:
+        def __init__(self, what):
+            self.what = what
+
+        def __enter__(self):
+            entered.append(self.what)
+
+        def __exit__(self, *exc):
+            left.append(self.what)
+
+    entered, left, s, dev = [], [], Stream(), torch.device("cuda", 0)
+    monkeypatch.setattr(api, "_raw_stream", None)
+    for name, f in (("current_device", lambda: 0), ("current_stream", lambda: s), ("device", Entered), ("stream", Entered)):
+        monkeypatch.setattr(torch.cuda, name, f)
+    with api._enqueue(dev, None) as handle:
+        assert handle == 77 and entered == [dev, s] and left == []
+    assert left == [s, dev]
