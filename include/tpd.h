@@ -319,7 +319,7 @@ tpd_status tpd_nonzero_write(const void* W, int n, int dtype, double tol, unsign
  *   values      device, nnz complex128.
  *   n           1..15.
  *   max_entries the most entries any level may hold (device memory grows with
- *               it: 80 bytes per entry); more sets *status to
+ *               it: 100 bytes per entry); more sets *status to
  *               TPD_ERR_WORKSPACE and the list is incomplete: what is left of the
  *               entries that fitted, sorted, *count <= max_entries of them.
  *               A level holds at most 2x the entries of the one before.

@@ -446,21 +446,25 @@ unsigned grid_for(unsigned long long items) {
 
 }  // namespace
 
-// Workspace: counters, X-mask maxima | two hash tables' keys | their values (two
-// slots an entry each: a level holds at most twice the entries of the one
-// before).  The last level leaves one table to be read and one free: the final
-// entries and their sort keys go into the free one's values (32 bytes an
-// entry, all of them), the second sort buffer into the other's, empty by then.
+// Workspace: counters, X-mask maxima | two hash tables' keys | their values.  A
+// level's table takes at most twice its entries; 2.5 slots an entry keep the
+// linear probes short (load 0.8; with two slots a level that just passes the
+// capacity fills its table: 10 times the time over attempts of growing
+// capacity).  The last level leaves one table to be read and one free: the
+// final entries and their sort keys go into the free one's values (32 of its 40
+// bytes an entry), the second sort buffer into the other's, empty by then.
 struct SparseLayout {
   size_t ctr, emax, tkeys, tvals, total;
-  unsigned long long entries, slots;
+  unsigned long long entries, slots, list;   // list: final entries there is room for (all, but for entries > 2^31)
 };
 
 static SparseLayout sparse_layout(unsigned long long max_entries) {
   auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
   SparseLayout L;
   L.entries = max_entries < 1 ? 1 : max_entries;
-  L.slots = 2 * L.entries;
+  L.slots = 2 * L.entries + L.entries / 2;
+  if (L.slots > 0xFFFFFFFFull) L.slots = 0xFFFFFFFFull;      // (a matrix has at most 2^30 entries)
+  L.list = L.entries < L.slots / 2 ? L.entries : L.slots / 2;
   size_t off = 0;
   L.ctr = off; off += al(kSpCounters * sizeof(unsigned long long));
   L.emax = off; off += al(sizeof(int) << 15);     // one per X-mask, n <= 15
@@ -509,19 +513,19 @@ cudaError_t launch_sparse(const int* rows, const int* cols, const void* vals, un
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const int lastt = (n - 1) & 1;                   // the last level's table; the other one is free
   longlong2* v = reinterpret_cast<longlong2*>(tv[lastt ^ 1]);
-  unsigned long long* skey = reinterpret_cast<unsigned long long*>(v + L.entries);
-  uint32_t* keys = reinterpret_cast<uint32_t*>(skey + L.entries);
-  uint32_t* sidx = keys + L.entries;
+  unsigned long long* skey = reinterpret_cast<unsigned long long*>(v + L.list);
+  uint32_t* keys = reinterpret_cast<uint32_t*>(skey + L.list);
+  uint32_t* sidx = keys + L.list;
   unsigned long long* skey2 = tv[lastt];           // once k_sp_final has read it
-  uint32_t* sidx2 = reinterpret_cast<uint32_t*>(skey2 + L.entries);
-  k_sp_final<<<tgrid, kSpThreads, 0, s>>>(tkeys[lastt], tv[lastt], slots, ctr, cap, n, keys, v, skey, sidx);
-  const unsigned chunks = (unsigned)((L.entries + kSpChunk - 1) / kSpChunk);
-  k_sp_local<<<chunks, kSpLocalThreads, 0, s>>>(skey, sidx, ctr, n, cap);
+  uint32_t* sidx2 = reinterpret_cast<uint32_t*>(skey2 + L.list);
+  k_sp_final<<<tgrid, kSpThreads, 0, s>>>(tkeys[lastt], tv[lastt], slots, ctr, L.list, n, keys, v, skey, sidx);
+  const unsigned chunks = (unsigned)((L.list + kSpChunk - 1) / kSpChunk);
+  k_sp_local<<<chunks, kSpLocalThreads, 0, s>>>(skey, sidx, ctr, n, L.list);
   int at = 0;
-  for (unsigned long long h = kSpChunk; h < L.entries; h <<= 1, at ^= 1)
-    k_sp_merge<<<grid_for(L.entries), 256, 0, s>>>(at ? skey2 : skey, at ? sidx2 : sidx, at ? skey : skey2,
-                                                   at ? sidx : sidx2, ctr, n, cap, h);
-  k_sp_emit<<<grid_for(cap), 256, 0, s>>>(keys, v, ctr, cap, skey, sidx, skey2, sidx2, n, emax, capacity, strings,
+  for (unsigned long long h = kSpChunk; h < L.list; h <<= 1, at ^= 1)
+    k_sp_merge<<<grid_for(L.list), 256, 0, s>>>(at ? skey2 : skey, at ? sidx2 : sidx, at ? skey : skey2,
+                                                at ? sidx : sidx2, ctr, n, L.list, h);
+  k_sp_emit<<<grid_for(L.list), 256, 0, s>>>(keys, v, ctr, L.list, skey, sidx, skey2, sidx2, n, emax, capacity, strings,
                                           static_cast<double2*>(weights), count, status);
   return cudaGetLastError();
 }
