@@ -168,7 +168,8 @@ tpd_status tpd_compose(void* C, int n, int dtype, double scale, const tpd_option
  * (device, only read) and leaving the result in another buffer (device, N*N
  * elements; its contents on entry are ignored).  The first pass reads the one
  * and writes the other, so no copy is made: a plan of P passes moves the
- * matrix P times each way instead of P + 1.  Input and output have the
+ * matrix P times each way instead of P + 1 (zero skipping outside the
+ * complex128 block fixed point copies the input first).  Input and output have the
  * alignment of tpd_decompose and are either the same buffer (then as in
  * place) or do not overlap (INVALID_ARG otherwise).  Results are those of the
  * in-place call on a copy, bit for bit.  Other arguments and errors as
@@ -369,7 +370,8 @@ tpd_status tpd_decompose_coo(const int* rows, const int* cols, const void* value
  *           complex64: fp32, rounded every level (FIXED and COMPENSATED are
  *           INVALID_ARG for complex64, FIXED for d = 5).
  * One kernel launch per pass of up to 4, 3, 2, 2 levels for d = 2, 3, 4,
- * 5 (block fixed point, d = 3: 2 levels; complex128 in IEEE fp64: per level).  No workspace; asynchronous on `stream`.
+ * 5 (block fixed point, d = 3: 2 levels; complex128 in IEEE fp64: per level).
+ * No workspace; asynchronous on `stream`.
  * Errors: INVALID_ARG, MISALIGNED, CUDA. */
 tpd_status tpd_weyl_decompose(void* A, int n, int d, int dtype, const tpd_options* opt, void* stream);
 

@@ -27,11 +27,11 @@
 // On the GPU every level is applied to all blocks at once.  complex128: one
 // launch per qudit, each thread one block of d^2 elements held in registers,
 // a grid-stride loop (bound by the fp64 pipe, so fusing levels would not help).
-// complex64: several levels per pass (tpd_qudit.cuh).  Arithmetic: IEEE fp64 (complex128) or fp32 (complex64),
-// rounded every level, without contraction into fused multiply-adds, so real
-// and imaginary parts see the same operations: conjugate blocks of a
-// Hermitian input stay exact conjugates level by level, and its
-// coefficients come out exactly real.
+// complex64: several levels per pass (tpd_gellmann_c64.cu).  Arithmetic: IEEE
+// fp64 (complex128) or fp32 (complex64), rounded every level, without
+// contraction into fused multiply-adds, so real and imaginary parts see the
+// same operations: conjugate blocks of a Hermitian input stay exact conjugates
+// level by level, and its coefficients come out exactly real.
 #include <cuda_runtime.h>
 #include <stdint.h>
 

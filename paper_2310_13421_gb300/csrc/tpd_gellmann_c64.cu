@@ -243,7 +243,7 @@ First first() {
 }
 
 // The first pass's kernel: as many column groups as the matrix has (up = n - K
-// digits above), up to 52 KB tiles (four CTAs an SM).
+// digits above), up to 52 KB tiles (three CTAs an SM, as for the later passes).
 template <bool kDec>
 First pick_first(int d, int K, int up) {
   switch (d * 8 + K) {

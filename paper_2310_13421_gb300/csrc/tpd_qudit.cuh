@@ -1,6 +1,6 @@
 // Several qudit levels of a complex64 Weyl-basis decomposition (or composition)
-// in one pass over the matrix (tpd_weyl_c64.cu), and the split of n levels into
-// passes that the other qudit kernels share.
+// in one pass over the matrix (tpd_weyl_c64.cu), and the levels per pass
+// that the other qudit kernels share.
 //
 // A level acts on every d x d block of one qudit's row and column digits,
 // all other digits fixed, and the levels of different qudits commute.  A pass
@@ -140,7 +140,8 @@ QuditKernel<Op> qudit_kernel() {
 }
 
 // Levels per pass at most: tiles of up to 52 KB (d = 3: 27 x 27 x 9) with the
-// longest runs that leave four CTAs an SM.
+// longest runs that leave four CTAs an SM.  (The complex64 Gell-Mann passes
+// follow it; the block fixed point has fixed_max_levels, tpd_weyl_fixed.cu.)
 constexpr int qudit_max_levels(int d) { return d == 2 ? 4 : (d == 3 ? 3 : 2); }
 
 // The kernel of a pass of K levels from level k0 of n: the most columns
